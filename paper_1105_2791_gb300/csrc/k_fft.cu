@@ -357,7 +357,8 @@ k_ring_c2r(int L, int R, int R_half, int RH, const float2* __restrict__ delta, c
 // grid: (ceil(R_half / RPB), nmp).  ut layout [nmp][L+1][2][RH].  If amax is not null,
 // amax[row / P] is raised (atomicMax on the float bits) to the largest |Re| or |Im| this
 // CTA writes: with amax cleared beforehand, it ends up as each map's max over all rows.
-template <int LOG2N>
+// WPIX: `ring_weight` holds a weight per pixel ([R][N]) instead of one per ring.
+template <int LOG2N, bool WPIX>
 __global__ void __launch_bounds__(FFT_THREADS, 2)
 k_ring_r2c(int L, int R, int R_half, int RH, int P, const float* __restrict__ maps,
            const float* __restrict__ ring_weight, const float4* __restrict__ tw, float2* __restrict__ ut,
@@ -379,11 +380,20 @@ k_ring_r2c(int L, int R, int R_half, int RH, int P, const float* __restrict__ ma
         const bool valid = q < ntr, south = valid && js != jn;
         const float* in_n = maps + ((int64_t)mp * R + (valid ? jn : 0)) * N;
         const float* in_s = maps + ((int64_t)mp * R + (south ? js : 0)) * N;
-        const float wn = (ring_weight && valid) ? ring_weight[jn] : 1.f;
-        const float ws = (ring_weight && south) ? ring_weight[js] : 1.f;
-        fft_passes_in<-1, N>(buf + q * NP, tl, tw, [&](int k) {
-            return make_float2(valid ? wn * __ldg(in_n + k) : 0.f, south ? ws * __ldg(in_s + k) : 0.f);
-        });
+        if constexpr (WPIX) {
+            const float* wn = ring_weight + (int64_t)(valid ? jn : 0) * N;
+            const float* ws = ring_weight + (int64_t)(south ? js : 0) * N;
+            fft_passes_in<-1, N>(buf + q * NP, tl, tw, [&](int k) {
+                return make_float2(valid ? __ldg(wn + k) * __ldg(in_n + k) : 0.f,
+                                   south ? __ldg(ws + k) * __ldg(in_s + k) : 0.f);
+            });
+        } else {
+            const float wn = (ring_weight && valid) ? ring_weight[jn] : 1.f;
+            const float ws = (ring_weight && south) ? ring_weight[js] : 1.f;
+            fft_passes_in<-1, N>(buf + q * NP, tl, tw, [&](int k) {
+                return make_float2(valid ? wn * __ldg(in_n + k) : 0.f, south ? ws * __ldg(in_s + k) : 0.f);
+            });
+        }
     }
     float2* o = ut + (int64_t)mp * (L + 1) * 2 * RH + j0;
     const int nout = (L + 1) << lgR;
@@ -429,17 +439,17 @@ static cudaError_t c2r_n(const Plan& pl, const float2* delta, int nmp, float* ma
     return cudaGetLastError();
 }
 
-template <int LOG2N>
+template <int LOG2N, bool WPIX>
 static cudaError_t r2c_n(const Plan& pl, const float* maps, int nmp, const float* ring_weight, float2* ut,
                          unsigned* amax, cudaStream_t st) {
     constexpr int N = 1 << LOG2N;
     const size_t smem = fft_smem(N);
-    cudaError_t e = cudaFuncSetAttribute(k_ring_r2c<LOG2N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_ring_r2c<LOG2N, WPIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int RPB = fft_rings_per_block(N);
     dim3 grid((pl.R_half + RPB - 1) / RPB, nmp);
-    k_ring_r2c<LOG2N><<<grid, FFT_THREADS, smem, st>>>(pl.lmax, pl.nrings, pl.R_half, pl.RH, pl.P, maps,
-                                                        ring_weight, pl.twiddle, ut, amax);
+    k_ring_r2c<LOG2N, WPIX><<<grid, FFT_THREADS, smem, st>>>(pl.lmax, pl.nrings, pl.R_half, pl.RH, pl.P, maps,
+                                                              ring_weight, pl.twiddle, ut, amax);
     note_launch(pl);
     return cudaGetLastError();
 }
@@ -461,22 +471,33 @@ cudaError_t launch_ring_c2r(const Plan& pl, const float2* delta, int nmp, float*
     }
 }
 
-cudaError_t launch_ring_r2c(const Plan& pl, const float* maps, int nmp, const float* ring_weight, float2* ut,
-                            unsigned* amax, cudaStream_t st) {
+template <bool WPIX>
+static cudaError_t r2c_any(const Plan& pl, const float* maps, int nmp, const float* weight, float2* ut, unsigned* amax,
+                           cudaStream_t st) {
     if (nmp == 0) return cudaSuccess;
     switch (ilog2(pl.nphi)) {
-        case 4: return r2c_n<4>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 5: return r2c_n<5>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 6: return r2c_n<6>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 7: return r2c_n<7>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 8: return r2c_n<8>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 9: return r2c_n<9>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 10: return r2c_n<10>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 11: return r2c_n<11>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 12: return r2c_n<12>(pl, maps, nmp, ring_weight, ut, amax, st);
-        case 13: return r2c_n<13>(pl, maps, nmp, ring_weight, ut, amax, st);
+        case 4: return r2c_n<4, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 5: return r2c_n<5, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 6: return r2c_n<6, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 7: return r2c_n<7, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 8: return r2c_n<8, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 9: return r2c_n<9, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 10: return r2c_n<10, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 11: return r2c_n<11, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 12: return r2c_n<12, WPIX>(pl, maps, nmp, weight, ut, amax, st);
+        case 13: return r2c_n<13, WPIX>(pl, maps, nmp, weight, ut, amax, st);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_ring_r2c(const Plan& pl, const float* maps, int nmp, const float* ring_weight, float2* ut,
+                            unsigned* amax, cudaStream_t st) {
+    return r2c_any<false>(pl, maps, nmp, ring_weight, ut, amax, st);
+}
+
+cudaError_t launch_ring_r2c_weighted(const Plan& pl, const float* rows, int nrows, const float* pix_weight, float2* ut,
+                                     cudaStream_t st) {
+    return r2c_any<true>(pl, rows, nrows, pix_weight, ut, nullptr, st);
 }
 
 }  // namespace modal

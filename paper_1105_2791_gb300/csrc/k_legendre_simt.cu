@@ -101,85 +101,176 @@ cudaError_t launch_legendre_simt(const Plan& pl, const float2* alm, int B, float
 //   rowfilt != NULL:  c_m sum_t rowfilt[t][l] G_t   (adjoint: c_0 = 1, c_m = 2)
 //   rowfilt == NULL:  G_0                           (quadrature analysis, nt = 1)
 // ut layout: [B][nt][lmax+1][2][RH] complex.
-template <int PM>
-__global__ void __launch_bounds__(128)
-k_legendre_adj_simt(int L, int nt, int R_half, int RH, const float* __restrict__ lam,
-                    const float2* __restrict__ ut, const float* __restrict__ rowfilt, int64_t n_alm,
-                    float2* __restrict__ out) {
-    constexpr int JT = 32;
-    __shared__ float sl[128][JT + 1];
-    __shared__ float2 su[PM][2][JT + 1];
-    const int m = blockIdx.y, b = blockIdx.z;
-    const int l0 = m + blockIdx.x * 128;
-    if (l0 > L) return;
-    const int nl = min(128, L + 1 - l0);
-    const int tid = threadIdx.x;
-    const int l = l0 + tid;
-    const int par = (l - m) & 1;
-    const int64_t base = d_alm_index(m, m, L);
-    const float* lrow = lam + (base + (l0 - m)) * (int64_t)RH;
-    const float2* ub = ut + ((int64_t)b * nt * (L + 1) + m) * 2 * RH;   // + t*(L+1)*2*RH + par*RH + j
+//
+// For one order and parity this is a GEMM: rows = values of l, columns = channels (map, t)
+// x (Re, Im), K = ring pairs, bound by FP32 arithmetic from about ten channels on and by the
+// read of the lambda table below.  A block holds LA_BM rows x NC channels, so that a row of
+// the table is read once per NC channels, and each thread TL rows x TC channels in
+// registers.  Both operands are contiguous along K in memory and stay so in shared memory
+// (cp.async, three stages of LA_BK ring pairs; a thread reads 16 bytes along K of each of its
+// rows and channels; the odd multiples of 16 bytes between rows keep the reads of a warp on
+// different banks).  Every output is one chain of FMAs over j ascending, whatever the tile.
+// 32 maps at l_max = 1000 (1001 x 2048): 8.80 ms with one channel per block (the table read
+// once per channel, three quarters of the arithmetic on padding), 0.70 ms now (46 TF/s, 0.58
+// of the measured FP32 rate); the 55 pair-mean rows at l_max = 500 2.06 -> 0.17 ms.
+constexpr int LA_BM = 64;                   // values of l (one parity) per block
+constexpr int LA_BK = 16;                   // ring pairs per stage
+constexpr int LA_STAGES = 3;
+constexpr int LA_SL = LA_BK + 4;            // floats per row of the lambda tile
+constexpr int LA_SU = 2 * LA_BK + 4;        // floats per channel of the U tile
 
-    float2 acc[PM];
-#pragma unroll
-    for (int t = 0; t < PM; ++t) acc[t] = make_float2(0.f, 0.f);
-
-    const int warp = tid >> 5, lane = tid & 31;
-    for (int j0 = 0; j0 < R_half; j0 += JT) {
-        __syncthreads();
-        for (int r = warp; r < 128; r += 4)
-            sl[r][lane] = (r < nl && j0 + lane < R_half) ? lrow[(int64_t)r * RH + j0 + lane] : 0.f;
-        for (int i = tid; i < PM * 2 * JT; i += 128) {
-            const int t = i / (2 * JT), pj = i % (2 * JT), pr = pj / JT, jj = pj % JT;
-            su[t][pr][jj] = (t < nt && j0 + jj < R_half)
-                                ? ub[((int64_t)t * (L + 1)) * 2 * RH + (int64_t)pr * RH + j0 + jj]
-                                : make_float2(0.f, 0.f);
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int jj = 0; jj < JT; ++jj) {
-            const float lv = sl[tid][jj];
-#pragma unroll
-            for (int t = 0; t < PM; ++t) {
-                const float2 u = su[t][par][jj];
-                acc[t].x = fmaf(lv, u.x, acc[t].x);
-                acc[t].y = fmaf(lv, u.y, acc[t].y);
-            }
-        }
-    }
-    if (tid >= nl) return;
-    float2 r = make_float2(0.f, 0.f);
-    if (rowfilt) {
-#pragma unroll
-        for (int t = 0; t < PM; ++t) {
-            if (t < nt) {
-                const float f = rowfilt[(int64_t)t * (L + 1) + l];
-                r.x = fmaf(f, acc[t].x, r.x);
-                r.y = fmaf(f, acc[t].y, r.y);
-            }
-        }
-        const float cm = (m == 0) ? 1.f : 2.f;
-        r.x *= cm;
-        r.y *= cm;
-        if (m == 0) r.y = 0.f;
-    } else {
-        r = acc[0];
-    }
-    out[(int64_t)b * n_alm + base + (l - m)] = r;
+__device__ __forceinline__ void la_cp16(float* dst, const void* src, int bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
 }
 
+template <int NC, int TL, int TC>
+__global__ void __launch_bounds__((LA_BM / TL) * (NC / TC))
+k_legendre_adj_simt(int L, int nt, int nchan, int cpb, int R_half, int RH, const float* __restrict__ lam,
+                    const float2* __restrict__ ut, const float* __restrict__ rowfilt, int64_t n_alm,
+                    float2* __restrict__ out) {
+    constexpr int NT = (LA_BM / TL) * (NC / TC);
+    constexpr int NLG = LA_BM / TL, NCG = NC / TC;           // thread groups along l and channels
+    constexpr int STAGE = LA_BM * LA_SL + NC * LA_SU;
+    __shared__ __align__(16) float sm[LA_STAGES * STAGE];
+    const int m = blockIdx.y >> 1, par = blockIdx.y & 1;
+    const int nl = (L - m - par >= 0) ? (L - m - par) / 2 + 1 : 0;     // rows of this order and parity
+    const int r0 = blockIdx.x * LA_BM;
+    if (r0 >= nl) return;
+    const int c0 = blockIdx.z * cpb;                          // first channel; cpb <= NC channels per block
+    const int nc = min(cpb, nchan - c0);
+    const int tid = threadIdx.x;
+    // half a warp holds 4 x CW threads, so that its 16-byte reads touch few rows and channels
+    constexpr int CW = NCG < 4 ? NCG : 4;
+    const int rest = tid / (4 * CW);
+    const int lg = tid % 4 + 4 * (rest % (NLG / 4));          // rows lg + NLG i
+    const int cg = (tid / 4) % CW + CW * (rest / (NLG / 4));  // channels cg + NCG k
+    const int64_t base = d_alm_index(m, m, L) + par;
+    const int64_t urow = (int64_t)(L + 1) * 2 * RH;           // ut stride between channels
+    const float2* ub = ut + (int64_t)c0 * urow + ((int64_t)m * 2 + par) * RH;
+
+    auto issue = [&](int k) {
+        const int j0 = k * LA_BK;
+        if (j0 < R_half) {
+            float* sl = sm + (k % LA_STAGES) * STAGE;
+            float* su = sl + LA_BM * LA_SL;
+#pragma unroll
+            for (int i = tid; i < LA_BM * (LA_BK / 4); i += NT) {
+                const int r = i / (LA_BK / 4), q = i % (LA_BK / 4);
+                const bool in = r0 + r < nl;                  // the table's row is zero from R_half to RH
+                la_cp16(sl + r * LA_SL + 4 * q, lam + (base + 2 * (int64_t)(in ? r0 + r : 0)) * RH + j0 + 4 * q, in ? 16 : 0);
+            }
+#pragma unroll
+            for (int i = tid; i < NC * (LA_BK / 2); i += NT) {
+                const int c = i / (LA_BK / 2), q = i % (LA_BK / 2);
+                const int left = (c < nc) ? R_half - (j0 + 2 * q) : 0;   // valid ring pairs of this 16-byte piece
+                la_cp16(su + c * LA_SU + 4 * q, ub + (left > 0 ? c * urow + j0 + 2 * q : 0), left >= 2 ? 16 : (left == 1 ? 8 : 0));
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    float2 acc[TL][TC];
+#pragma unroll
+    for (int i = 0; i < TL; ++i)
+#pragma unroll
+        for (int k = 0; k < TC; ++k) acc[i][k] = make_float2(0.f, 0.f);
+    const int nk = (R_half + LA_BK - 1) / LA_BK;
+#pragma unroll
+    for (int k = 0; k < LA_STAGES - 1; ++k) issue(k);
+    for (int k = 0; k < nk; ++k) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(LA_STAGES - 2) : "memory");
+        __syncthreads();                                      // stage k is here, stage k - 1 is free
+        issue(k + LA_STAGES - 1);
+        const float* sl = sm + (k % LA_STAGES) * STAGE + lg * LA_SL;
+        const float* su = sm + (k % LA_STAGES) * STAGE + LA_BM * LA_SL + cg * LA_SU;
+#pragma unroll
+        for (int q = 0; q < LA_BK / 4; ++q) {
+            float4 lv[TL];
+#pragma unroll
+            for (int i = 0; i < TL; ++i) lv[i] = *reinterpret_cast<const float4*>(sl + i * NLG * LA_SL + 4 * q);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float4 uv[TC];
+#pragma unroll
+                for (int c = 0; c < TC; ++c) uv[c] = *reinterpret_cast<const float4*>(su + c * NCG * LA_SU + 8 * q + 4 * h);
+#pragma unroll
+                for (int i = 0; i < TL; ++i) {
+                    const float l0 = h ? lv[i].z : lv[i].x, l1 = h ? lv[i].w : lv[i].y;
+                    const float2 l02 = make_float2(l0, l0), l12 = make_float2(l1, l1);
+#pragma unroll
+                    for (int c = 0; c < TC; ++c) acc[i][c] = __ffma2_rn(l02, make_float2(uv[c].x, uv[c].y), acc[i][c]);
+#pragma unroll
+                    for (int c = 0; c < TC; ++c) acc[i][c] = __ffma2_rn(l12, make_float2(uv[c].z, uv[c].w), acc[i][c]);
+                }
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!rowfilt) {
+#pragma unroll
+        for (int i = 0; i < TL; ++i)
+#pragma unroll
+            for (int c = 0; c < TC; ++c) {
+                const int r = r0 + lg + NLG * i, ch = cg + NCG * c;
+                if (r < nl && ch < nc) out[(int64_t)(c0 + ch) * n_alm + base + 2 * r] = acc[i][c];
+            }
+        return;
+    }
+    // the nt channels of each map meet in shared memory: one thread per (row, map) sums them
+    __syncthreads();
+    float2* g = reinterpret_cast<float2*>(sm);                // [LA_BM][NC + 1]
+    static_assert(LA_BM * (NC + 1) * 2 <= LA_STAGES * STAGE, "the G tile fits the stages");
+#pragma unroll
+    for (int i = 0; i < TL; ++i)
+#pragma unroll
+        for (int c = 0; c < TC; ++c) g[(lg + NLG * i) * (NC + 1) + cg + NCG * c] = acc[i][c];
+    __syncthreads();
+    for (int i = tid; i < LA_BM * (nc / nt); i += NT) {
+        const int r = i % LA_BM, b = i / LA_BM;
+        if (r0 + r >= nl) continue;
+        const int l = m + par + 2 * (r0 + r);
+        float2 v = make_float2(0.f, 0.f);
+        for (int t = 0; t < nt; ++t) {
+            const float f = rowfilt[(int64_t)t * (L + 1) + l];
+            const float2 a = g[r * (NC + 1) + b * nt + t];
+            v.x = fmaf(f, a.x, v.x);
+            v.y = fmaf(f, a.y, v.y);
+        }
+        const float cm = (m == 0) ? 1.f : 2.f;
+        v.x *= cm;
+        v.y *= cm;
+        if (m == 0) v.y = 0.f;
+        out[(int64_t)(c0 / nt + b) * n_alm + base + 2 * (r0 + r)] = v;
+    }
+}
+
+template <int NC, int TL, int TC>
+static cudaError_t legendre_adj_launch(const Plan& pl, const float2* ut, int B, const float* rowfilt, int nt,
+                                       float2* out, cudaStream_t st) {
+    const int nchan = B * nt;
+    const int cpb = rowfilt ? NC / nt * nt : NC;               // whole maps per block where their channels are summed
+    const int nlmax = pl.lmax / 2 + 1;
+    const dim3 grid((nlmax + LA_BM - 1) / LA_BM, 2 * (pl.lmax + 1), (nchan + cpb - 1) / cpb);
+    k_legendre_adj_simt<NC, TL, TC><<<grid, (LA_BM / TL) * (NC / TC), 0, st>>>(
+        pl.lmax, nt, nchan, cpb, pl.R_half, pl.RH, pl.lam, ut, rowfilt, pl.n_alm, out);
+    note_launch(pl);
+    return cudaGetLastError();
+}
+
+// ut: nt channels for each of B maps.  Without rowfilt the channels are independent rows (nt = 1).
 cudaError_t launch_legendre_adjoint_simt(const Plan& pl, const float2* ut, int B, const float* rowfilt,
                                          int nt, float2* out, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
-    dim3 grid((pl.lmax + 1 + 127) / 128, pl.lmax + 1, B);
-    note_launch(pl);
-    if (nt <= 4)
-        k_legendre_adj_simt<4><<<grid, 128, 0, st>>>(pl.lmax, nt, pl.R_half, pl.RH, pl.lam, ut, rowfilt, pl.n_alm, out);
-    else if (nt <= 8)
-        k_legendre_adj_simt<8><<<grid, 128, 0, st>>>(pl.lmax, nt, pl.R_half, pl.RH, pl.lam, ut, rowfilt, pl.n_alm, out);
-    else
-        k_legendre_adj_simt<16><<<grid, 128, 0, st>>>(pl.lmax, nt, pl.R_half, pl.RH, pl.lam, ut, rowfilt, pl.n_alm, out);
-    return cudaGetLastError();
+    if (nt < 1 || nt > MODAL_MAXP || (!rowfilt && nt != 1)) return cudaErrorInvalidValue;
+    // the narrowest tile that holds the channels of the call, so that little work goes to padding
+    // (l_max = 1000, us for 1, 2 / 4, 8 / 16 / 32 channels: 169, 173 / 252, 254 / 418 / 715; with
+    // the 32-channel tile alone every call takes the last time)
+    const int nchan = B * nt;
+    if (nchan > 16) return legendre_adj_launch<32, 8, 4>(pl, ut, B, rowfilt, nt, out, st);
+    if (nchan > 8) return legendre_adj_launch<16, 8, 2>(pl, ut, B, rowfilt, nt, out, st);
+    if (nchan > 2) return legendre_adj_launch<8, 4, 2>(pl, ut, B, rowfilt, nt, out, st);
+    return legendre_adj_launch<2, 2, 1>(pl, ut, B, rowfilt, nt, out, st);
 }
 
 }  // namespace modal

@@ -39,25 +39,27 @@ constexpr int LH_APT = (LH_MAPS * LH_MC + LH_THREADS - 1) / LH_THREADS;  // a_lm
 
 __host__ __device__ inline int64_t av_lidx(int64_t l, int64_t m) { return l * (l + 1) / 2 + m; }
 
-// in[c][x] = W_x <c>_x
-__global__ void k_adjpm_weighted(int64_t npix, int n_pair, const float* __restrict__ W, const float* __restrict__ pm,
-                                 float* __restrict__ out) {
-    const int64_t n = (int64_t)n_pair * npix;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = W[i % npix] * pm[i];
-}
-
-// F[c][l (l+1)/2 + m] = in[c][alm index (l, m)]: the l-major copy read by k_adjpm_grad
-__global__ void k_adjpm_lmajor(int L, int64_t n_alm, const float2* __restrict__ in, float2* __restrict__ F) {
-    const int c = blockIdx.y;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_alm; i += (int64_t)gridDim.x * blockDim.x) {
-        // i = m (2 L + 3 - m) / 2 + (l - m): recover m by the closed form, then correct by one
-        int m = (int)((2.0 * L + 3.0 - sqrt((2.0 * L + 3.0) * (2.0 * L + 3.0) - 8.0 * (double)i)) / 2.0);
-        m = max(0, min(L, m));
-        while (m > 0 && d_alm_index(m, m, L) > i) --m;
-        while (m < L && d_alm_index(m + 1, m + 1, L) <= i) ++m;
-        const int l = m + (int)(i - d_alm_index(m, m, L));
-        F[(int64_t)c * n_alm + av_lidx(l, m)] = in[(int64_t)c * n_alm + i];
+// F[c][l (l+1)/2 + m] = in[c][alm index (l, m)]: the l-major table, through 32 x 32 tiles of
+// (l, m) in shared memory so that `in` is read contiguous in l and F written contiguous in m
+// (one value per thread with F written in scattered 8-byte pieces took 195 us for 55 rows at
+// l_max = 500).
+__global__ void __launch_bounds__(256) k_adjpm_lmajor(int L, int64_t n_alm, const float2* __restrict__ in,
+                                                      float2* __restrict__ F) {
+    __shared__ float2 tile[32][33];
+    const int nlb = (L + 32) / 32;
+    const int lb = blockIdx.x / nlb, mb = blockIdx.x % nlb;
+    if (mb > lb) return;
+    const float2* src = in + (int64_t)blockIdx.y * n_alm;
+    float2* dst = F + (int64_t)blockIdx.y * n_alm;
+    const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+    for (int j = ty; j < 32; j += 8) {                     // row m = 32 mb + j, column l = 32 lb + tx
+        const int m = 32 * mb + j, l = 32 * lb + tx;
+        if (l <= L && m <= l) tile[tx][j] = src[d_alm_index(l, m, L)];
+    }
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8) {                     // row l = 32 lb + i, column m = 32 mb + tx
+        const int l = 32 * lb + i, m = 32 * mb + tx;
+        if (l <= L && m <= l) dst[av_lidx(l, m)] = tile[i][tx];
     }
 }
 
@@ -85,33 +87,28 @@ cudaError_t build_pm_table(Plan& pl, cudaStream_t st) {
         e = cudaMemcpy(pl.adj_pm_blk, blk.data(), blk.size() * sizeof(int), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return e;
     }
-    const size_t L1 = pl.lmax + 1;
-    float* win = nullptr;
-    float2* ut = nullptr;
-    float2* fm = nullptr;
-    cudaError_t e = cudaMallocAsync(&win, (size_t)pl.n_pair * pl.npix * sizeof(float), st);
-    if (e == cudaSuccess) e = cudaMallocAsync(&ut, (size_t)pl.n_pair * L1 * 2 * pl.RH * sizeof(float2), st);
-    if (e == cudaSuccess) e = cudaMallocAsync(&fm, (size_t)pl.n_pair * pl.n_alm * sizeof(float2), st);
-    if (e == cudaSuccess) {
-        k_adjpm_weighted<<<pl.nsm * 8, 256, 0, st>>>(pl.npix, pl.n_pair, pl.W, pl.pair_mean, win);
+    // the adjoint's own transforms without the filter: ring r2c of the rows W<c> (the pixel
+    // weight applied as the rows are read, no ring weights), then the transposed Legendre sums
+    // of each row.  The rows go through the plan's Fourier and Legendre workspaces, as many at
+    // a time as these hold (chunk P >= n_pair in all but the smallest workspaces): neither
+    // holds anything that a later call reads, and a Legendre row of 2 (lmax + 1) RH values is
+    // longer than n_alm.
+    const int rows = (int)std::min<int64_t>((int64_t)pl.chunk * pl.P, pl.n_pair);
+    if (rows < 1 || !pl.ut || !pl.delta) return cudaErrorInvalidValue;
+    const int nlb = (pl.lmax + 32) / 32;
+    for (int c0 = 0; c0 < pl.n_pair; c0 += rows) {
+        const int n = std::min(rows, pl.n_pair - c0);
+        cudaError_t e = launch_ring_r2c_weighted(pl, pl.pair_mean + (int64_t)c0 * pl.npix, n, pl.W, pl.ut, st);
+        if (e == cudaSuccess) e = launch_legendre_adjoint_simt(pl, pl.ut, n, nullptr, 1, pl.delta, st);
+        if (e != cudaSuccess) return e;
+        k_adjpm_lmajor<<<dim3(nlb * nlb, n), 256, 0, st>>>(pl.lmax, pl.n_alm, pl.delta,
+                                                           pl.adj_pm + (int64_t)c0 * pl.n_alm);
         note_launch(pl);
         e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
     }
-    // the adjoint's own transforms without the filter: ring r2c (no ring weights: W is in
-    // the rows), then the transposed Legendre sums of each row
-    if (e == cudaSuccess) e = launch_ring_r2c(pl, win, pl.n_pair, nullptr, ut, nullptr, st);
-    if (e == cudaSuccess) e = launch_legendre_adjoint_simt(pl, ut, pl.n_pair, nullptr, 1, fm, st);
-    if (e == cudaSuccess) {
-        k_adjpm_lmajor<<<dim3(std::max(1, std::min(pl.nsm * 2, (int)((pl.n_alm + 255) / 256))), pl.n_pair), 256, 0, st>>>(
-            pl.lmax, pl.n_alm, fm, pl.adj_pm);
-        note_launch(pl);
-        e = cudaGetLastError();
-    }
-    if (win) cudaFreeAsync(win, st);
-    if (ut) cudaFreeAsync(ut, st);
-    if (fm) cudaFreeAsync(fm, st);
-    if (e == cudaSuccess) pl.adj_pm_ready = 1;
-    return e;
+    pl.adj_pm_ready = 1;
+    return cudaSuccess;
 }
 
 // K[l][b][c] = sum_t f_t(l) h_{b,t,c}

@@ -195,6 +195,9 @@ cudaError_t launch_legendre_tc(const Plan& pl, const float2* alm, int B, float2*
 cudaError_t launch_ring_c2r(const Plan& pl, const float2* delta, int nmaps_p, float* maps, cudaStream_t st);
 cudaError_t launch_ring_r2c(const Plan& pl, const float* maps, int nmaps_p, const float* ring_weight,
                             float2* ut, unsigned* amax, cudaStream_t st);
+// the same transform of rows [nrows][npix], each pixel times pix_weight [npix] as it is read
+cudaError_t launch_ring_r2c_weighted(const Plan& pl, const float* rows, int nrows, const float* pix_weight, float2* ut,
+                                     cudaStream_t st);
 // k_cubic.cu
 cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st);
 // The cubic sums of B[i] maps (one chunk, at maps[i], partial sums into plan i's partial
