@@ -354,51 +354,267 @@ cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cu
 
 // ---------------------------------------------------------------- linear term GEMM
 // out[z][row][col] = sum_{x in split z} (W_x <pair row>_x) * maps[col][x],
-// rows = pairs (lexicographic), cols = (map, c) = b * P + c.  64 x 64 CTA tiles,
-// 4 x 4 register tiles, K (pixels) staged 32 at a time, split over gridDim.z.
-constexpr int LG_TM = 64, LG_TN = 64, LG_TK = 32;
+// rows = pairs (lexicographic), cols = (map, c) = b * P + c, K = pixels, split over gridDim.z.
+// Every output of a split is one chain of FMAs over its pixels in order, whatever the tile, so
+// a small problem is bound by that chain and by how many SMs its few outputs reach, a large
+// one by FP32 arithmetic.  Panel and maps are contiguous along K in memory and stay so in
+// shared memory: a ring of ST stages of BK pixels filled by cp.async, each thread multiplying
+// the panel pieces that it copied by W once they are there.  A thread reads 4 pixels (16
+// bytes) of its TL rows and TC columns at a time; the padding of 4 floats per row puts the
+// rows on different banks.  Synchronous staging through registers, one tile of 64 x 64 for
+// every size, took (us, linear term of one call) 290 at l_max = 32 with 6 modes and one map,
+// 2467 at l_max = 250 with 8 modes and 21 maps; now 28 and 183.
+__device__ __forceinline__ void lg_cp16(float* dst, const float* src, int bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
 
-__global__ void __launch_bounds__(256)
+template <int BM, int BN, int BK, int ST>
+constexpr size_t lg_smem() { return (size_t)ST * (BM + BN) * (BK + 4) * sizeof(float); }
+
+template <int BM, int BN, int TL, int TC, int BK, int ST>
+__global__ void __launch_bounds__((BM / TL) * (BN / TC))
 k_linear_gemm(int nrows, int ncols, int64_t npix, int64_t kchunk, const float* __restrict__ panel,
               const float* __restrict__ W, const float* __restrict__ maps, double* __restrict__ out) {
-    __shared__ __align__(16) float sA[LG_TK][LG_TM + 4];
-    __shared__ __align__(16) float sB[LG_TK][LG_TN + 4];
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const int r0 = blockIdx.x * LG_TM, c0 = blockIdx.y * LG_TN;
+    constexpr int NT = (BM / TL) * (BN / TC), S = BK + 4, Q = BK / 4;
+    constexpr int STAGE = (BM + BN) * S;
+    constexpr int NR = BM / TL, NCG = BN / TC;               // thread groups along rows and columns
+    constexpr int RS = NT / Q;                               // rows between a thread's copies
+    constexpr int NA = BM / RS, NB = BN / RS;                // its 16-byte pieces of the panel and of the maps per stage
+    static_assert(NT % Q == 0 && BM % RS == 0 && BN % RS == 0 && NR % 4 == 0 && NCG % 4 == 0, "tile shape");
+    extern __shared__ __align__(16) float lg_sm[];
+    const int tid = threadIdx.x;
+    // half a warp holds 4 x 4 threads, so that its 16-byte reads touch 4 rows and 4 columns
+    const int rg = tid % 4 + 4 * ((tid / 16) % (NR / 4)), cg = (tid / 4) % 4 + 4 * (tid / (4 * NR));
+    const int r0 = blockIdx.x * BM, c0 = blockIdx.y * BN;    // rows rg + NR i, columns cg + NCG k
+    const int64_t k_begin = (int64_t)blockIdx.z * kchunk;
+    const int64_t k_end = min(npix, k_begin + kchunk);       // a multiple of 16, as npix and kchunk are
+    const int nk = k_end > k_begin ? (int)((k_end - k_begin + BK - 1) / BK) : 0;
+    // this thread copies piece q of rows lr + RS u; a piece past the last pixel, row or column is zero
+    const int q = tid % Q, lr = tid / Q;
+    const float* pa = panel + (int64_t)(r0 + lr) * npix + k_begin + 4 * q;
+    const float* pb = maps + (int64_t)(c0 + lr) * npix + k_begin + 4 * q;
+    const float* pw = W + k_begin + 4 * q;
+    const int64_t step = (int64_t)RS * npix;
+    auto issue = [&](int k) {
+        if (k < nk) {
+            const int off = k * BK;
+            const bool in = k_begin + off + 4 * q < k_end;
+            float* st = lg_sm + (k % ST) * STAGE + lr * S + 4 * q;
+#pragma unroll
+            for (int u = 0; u < NA; ++u) {
+                const bool ok = in && r0 + lr + RS * u < nrows;
+                lg_cp16(st + RS * u * S, ok ? pa + off + u * step : panel, ok ? 16 : 0);
+            }
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+                const bool ok = in && c0 + lr + RS * u < ncols;
+                lg_cp16(st + (BM + RS * u) * S, ok ? pb + off + u * step : maps, ok ? 16 : 0);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto weight = [&](int k) {
+        return k < nk && k_begin + (int64_t)k * BK + 4 * q < k_end ? __ldg(reinterpret_cast<const float4*>(pw + k * BK))
+                                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    float acc[TL][TC];
+#pragma unroll
+    for (int i = 0; i < TL; ++i)
+#pragma unroll
+        for (int j = 0; j < TC; ++j) acc[i][j] = 0.f;
+#pragma unroll
+    for (int k = 0; k < ST - 1; ++k) issue(k);
+    float4 w = weight(0);
+    for (int k = 0; k < nk; ++k) {
+        const float4 wn = weight(k + 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(ST - 2) : "memory");
+        // the panel's pieces that this thread copied, times W
+        float* own = lg_sm + (k % ST) * STAGE + lr * S + 4 * q;
+#pragma unroll
+        for (int u = 0; u < NA; ++u) {
+            float4* v = reinterpret_cast<float4*>(own + RS * u * S);
+            const float4 x = *v;
+            *v = make_float4(x.x * w.x, x.y * w.y, x.z * w.z, x.w * w.w);
+        }
+        w = wn;
+        __syncthreads();                                     // stage k is ready, stage k - 1 is free
+        issue(k + ST - 1);
+        const float* sa = lg_sm + (k % ST) * STAGE + rg * S;
+        const float* sb = lg_sm + (k % ST) * STAGE + (BM + cg) * S;
+        constexpr int UNROLL = TL * TC >= 32 ? 2 : (TL * TC >= 16 ? 4 : 8);
+#pragma unroll UNROLL
+        for (int p = 0; p < Q; ++p) {
+            float4 a[TL], b[TC];
+#pragma unroll
+            for (int i = 0; i < TL; ++i) a[i] = *reinterpret_cast<const float4*>(sa + i * NR * S + 4 * p);
+#pragma unroll
+            for (int j = 0; j < TC; ++j) b[j] = *reinterpret_cast<const float4*>(sb + j * NCG * S + 4 * p);
+#pragma unroll
+            for (int i = 0; i < TL; ++i)
+#pragma unroll
+                for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < TL; ++i)
+#pragma unroll
+                for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < TL; ++i)
+#pragma unroll
+                for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < TL; ++i)
+#pragma unroll
+                for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < TL; ++i)
+#pragma unroll
+        for (int j = 0; j < TC; ++j) {
+            const int r = r0 + rg + NR * i, c = c0 + cg + NCG * j;
+            if (r < nrows && c < ncols) out[((int64_t)blockIdx.z * nrows + r) * ncols + c] = (double)acc[i][j];
+        }
+}
+
+template <int BM, int BN, int TL, int TC, int BK, int ST>
+static cudaError_t linear_gemm_launch(Plan& pl, const float* maps, int ncols, int64_t kchunk, double* partial,
+                                      cudaStream_t st) {
+    constexpr size_t smem = lg_smem<BM, BN, BK, ST>();
+    auto kernel = k_linear_gemm<BM, BN, TL, TC, BK, ST>;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    const dim3 grid((pl.n_pair + BM - 1) / BM, (ncols + BN - 1) / BN, pl.lin_ksplit);
+    kernel<<<grid, (BM / TL) * (BN / TC), smem, st>>>(pl.n_pair, ncols, pl.npix, kchunk, pl.pair_mean, pl.W, maps, partial);
+    note_launch(pl);
+    return cudaGetLastError();
+}
+
+// The same sums where the outputs are few: 16 x 16 outputs per block, 2 x 2 per thread of two
+// compute warps, which do nothing but read and accumulate (a stage of LC_BK pixels is 4 LC_BK
+// FMAs deep per chain); two copy warps keep LC_ST stages in flight and multiply the panel's
+// pieces by W.  With copies, weights and sums in the same warps the chain advanced by one
+// pixel in 20 cycles.  Blocks alternate which warps compute, so that the compute warps of two
+// blocks on an SM sit on different sub-partitions.
+constexpr int LC_BK = 64, LC_ST = 4, LC_S = LC_BK + 4, LC_Q = LC_BK / 4;
+constexpr int LC_G = 4;                     // pieces per read-ahead group
+constexpr int LC_STAGE = 32 * LC_S;
+constexpr size_t LC_SMEM = (size_t)LC_ST * LC_STAGE * sizeof(float);
+
+__global__ void __launch_bounds__(128)
+k_linear_chain(int nrows, int ncols, int64_t npix, int64_t kchunk, const float* __restrict__ panel,
+               const float* __restrict__ W, const float* __restrict__ maps, double* __restrict__ out) {
+    extern __shared__ __align__(16) float lg_sm[];
+    const int r0 = blockIdx.x * 16, c0 = blockIdx.y * 16;
     const int64_t k_begin = (int64_t)blockIdx.z * kchunk;
     const int64_t k_end = min(npix, k_begin + kchunk);
-    float acc[4][4] = {};
-    for (int64_t k0 = k_begin; k0 < k_end; k0 += LG_TK) {
-        for (int i = tid; i < LG_TM * LG_TK; i += 256) {
-            const int r = i / LG_TK, k = i % LG_TK;
-            const int64_t x = k0 + k;
-            float v = 0.f;
-            if (r0 + r < nrows && x < k_end) v = panel[(int64_t)(r0 + r) * npix + x] * W[x];
-            sA[k][r] = v;
-        }
-        for (int i = tid; i < LG_TN * LG_TK; i += 256) {
-            const int c = i / LG_TK, k = i % LG_TK;
-            const int64_t x = k0 + k;
-            sB[k][c] = (c0 + c < ncols && x < k_end) ? maps[(int64_t)(c0 + c) * npix + x] : 0.f;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int k = 0; k < LG_TK; ++k) {
-            const float4 a = *reinterpret_cast<const float4*>(&sA[k][ty * 4]);
-            const float4 bb = *reinterpret_cast<const float4*>(&sB[k][tx * 4]);
-            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
+    const int nk = k_end > k_begin ? (int)((k_end - k_begin + LC_BK - 1) / LC_BK) : 0;
+    const int swap = (blockIdx.x + blockIdx.y + blockIdx.z) & 1;
+    const int role = (threadIdx.x / 64) ^ swap;              // 0: compute, 1: copy
+    const int tid = threadIdx.x % 64;
+    // barriers: 1 + s: stage s is filled; 1 + LC_ST + s: stage s has been read
+    if (role == 1) {
+        const int q = tid % LC_Q, lr = tid / LC_Q;           // pieces q of rows lr + RS u
+        constexpr int RS = 64 / LC_Q, NU = 16 / RS;
+        const float* pa = panel + (int64_t)(r0 + lr) * npix + k_begin + 4 * q;
+        const float* pb = maps + (int64_t)(c0 + lr) * npix + k_begin + 4 * q;
+        const float* pw = W + k_begin + 4 * q;
+        const int64_t step = (int64_t)RS * npix;
+        float4 w[LC_ST];
+        auto issue = [&](int k, float4& wk) {
+            wk = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k < nk) {
+                const int off = k * LC_BK;
+                const bool in = k_begin + off + 4 * q < k_end;
+                float* st = lg_sm + (k % LC_ST) * LC_STAGE + lr * LC_S + 4 * q;
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+                for (int u = 0; u < NU; ++u) {
+                    const bool oka = in && r0 + lr + RS * u < nrows, okb = in && c0 + lr + RS * u < ncols;
+                    lg_cp16(st + RS * u * LC_S, oka ? pa + off + u * step : panel, oka ? 16 : 0);
+                    lg_cp16(st + (16 + RS * u) * LC_S, okb ? pb + off + u * step : maps, okb ? 16 : 0);
+                }
+                if (in) wk = __ldg(reinterpret_cast<const float4*>(pw + off));
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        for (int k = 0; k < LC_ST - 1; ++k) issue(k, w[k]);
+        for (int k0 = 0; k0 < nk; k0 += LC_ST) {
+#pragma unroll
+            for (int s = 0; s < LC_ST; ++s) {                // stage s holds step k
+                const int k = k0 + s;
+                if (k >= nk) break;
+                asm volatile("cp.async.wait_group %0;" ::"n"(LC_ST - 2) : "memory");
+                float* own = lg_sm + s * LC_STAGE + lr * LC_S + 4 * q;
+#pragma unroll
+                for (int u = 0; u < NU; ++u) {
+                    float4* v = reinterpret_cast<float4*>(own + RS * u * LC_S);
+                    const float4 x = *v;
+                    *v = make_float4(x.x * w[s].x, x.y * w[s].y, x.z * w[s].z, x.w * w[s].w);
+                }
+                __threadfence_block();
+                named_arrive(1 + s, 128);
+                const int kn = k + LC_ST - 1;                // goes where step k - 1 was
+                if (k >= 1 && kn < nk) named_sync(1 + LC_ST + (s + LC_ST - 1) % LC_ST, 128);
+                issue(kn, w[(s + LC_ST - 1) % LC_ST]);
+            }
         }
-        __syncthreads();
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        return;
+    }
+    const int rg = tid % 4 + 4 * ((tid / 16) % 2), cg = (tid / 4) % 4 + 4 * (tid / 32);   // rows rg, rg + 8; columns cg, cg + 8
+    float acc[2][2] = {};
+    for (int k = 0; k < nk; ++k) {
+        const int s = k % LC_ST;
+        named_sync(1 + s, 128);
+        const float* sa = lg_sm + s * LC_STAGE + rg * LC_S;
+        const float* sb = lg_sm + s * LC_STAGE + (16 + cg) * LC_S;
+        // groups of LC_G pieces: the next group's reads are issued before this group's sums
+        float4 a[2][LC_G][2], b[2][LC_G][2];
+        auto read = [&](int h, int g) {
+#pragma unroll
+            for (int p = 0; p < LC_G; ++p)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    a[h][p][i] = *reinterpret_cast<const float4*>(sa + 8 * i * LC_S + 4 * (g * LC_G + p));
+                    b[h][p][i] = *reinterpret_cast<const float4*>(sb + 8 * i * LC_S + 4 * (g * LC_G + p));
+                }
+        };
+        read(0, 0);
+#pragma unroll
+        for (int g = 0; g < LC_Q / LC_G; ++g) {
+            const int h = g & 1;
+            if (g + 1 < LC_Q / LC_G) read(h ^ 1, g + 1);
+#pragma unroll
+            for (int p = 0; p < LC_G; ++p) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[h][p][i].x, b[h][p][j].x, acc[i][j]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[h][p][i].y, b[h][p][j].y, acc[i][j]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[h][p][i].z, b[h][p][j].z, acc[i][j]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[h][p][i].w, b[h][p][j].w, acc[i][j]);
+            }
+        }
+        if (k + LC_ST < nk) named_arrive(1 + LC_ST + s, 128);    // the copy of step k + LC_ST waits for this
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = r0 + ty * 4 + i, c = c0 + tx * 4 + j;
+        for (int j = 0; j < 2; ++j) {
+            const int r = r0 + rg + 8 * i, c = c0 + cg + 8 * j;
             if (r < nrows && c < ncols) out[((int64_t)blockIdx.z * nrows + r) * ncols + c] = (double)acc[i][j];
         }
 }
@@ -406,9 +622,21 @@ k_linear_gemm(int nrows, int ncols, int64_t npix, int64_t kchunk, const float* _
 cudaError_t launch_linear_gemm(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
     const int ncols = B * pl.P;
-    const int64_t kchunk = ((pl.npix + pl.lin_ksplit - 1) / pl.lin_ksplit + LG_TK - 1) / LG_TK * LG_TK;
-    dim3 grid((pl.n_pair + LG_TM - 1) / LG_TM, (ncols + LG_TN - 1) / LG_TN, pl.lin_ksplit);
-    k_linear_gemm<<<grid, 256, 0, st>>>(pl.n_pair, ncols, pl.npix, kchunk, pl.pair_mean, pl.W, maps, partial);
+    const int64_t kchunk = ((pl.npix + pl.lin_ksplit - 1) / pl.lin_ksplit + 31) / 32 * 32;
+    auto blocks = [&](int bm, int bn) {
+        return (int64_t)((pl.n_pair + bm - 1) / bm) * ((ncols + bn - 1) / bn) * pl.lin_ksplit;
+    };
+    // The largest tile that still fills the SMs: a block of the larger tiles is two warps, and an
+    // SM needs about eight of them before its FP32 units are busy (136 pairs x 16 maps on 501 x
+    // 1024 pixels with one block per SM, us: 64 x 64 1507, 32 x 32 892); below two blocks of 32 x
+    // 32 per SM the chains' own latency is the bound (55 pairs, 8 maps of 10 modes: 452 with
+    // 32 x 32 tiles, 370 with k_linear_chain).
+    if (blocks(64, 64) >= 4 * (int64_t)pl.nsm) return linear_gemm_launch<64, 64, 8, 8, 16, 4>(pl, maps, ncols, kchunk, partial, st);
+    if (blocks(32, 32) >= 2 * (int64_t)pl.nsm) return linear_gemm_launch<32, 32, 4, 4, 32, 4>(pl, maps, ncols, kchunk, partial, st);
+    const cudaError_t e = cudaFuncSetAttribute(k_linear_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LC_SMEM);
+    if (e != cudaSuccess) return e;
+    k_linear_chain<<<dim3((pl.n_pair + 15) / 16, (ncols + 15) / 16, pl.lin_ksplit), 128, LC_SMEM, st>>>(
+        pl.n_pair, ncols, pl.npix, kchunk, pl.pair_mean, pl.W, maps, partial);
     note_launch(pl);
     return cudaGetLastError();
 }
