@@ -940,36 +940,88 @@ static modal_status read_device_error(modal_h h, cudaStream_t st, int* word) {
     return MODAL_OK;
 }
 
+// The FP64 workspace of one modal_solve or modal_fnl_weights call: zeta and its factor, the
+// carried rows (alpha, betas), the diagonal-block scratch and the results with the error word.
+// Up to kSolveKeep carried rows it is the plan's own, allocated by the first such call (both
+// calls synchronise, so one plan never needs two); a larger batch allocates for the call.
+constexpr int kSolveKeep = 257;
+
+struct SolveSpace {
+    double *A = nullptr, *rows = nullptr, *diag = nullptr, *est = nullptr;
+    double* owned = nullptr;                       // allocated for this call alone
+};
+
+static size_t solve_doubles(size_t n, size_t rows) { return n * n + rows * n + CHOL_DIAG + rows + 1; }
+
+static modal_status solve_space(modal_h h, int nrows, cudaStream_t st, SolveSpace* sp) {
+    const size_t n = h->n_max;
+    double* ws = nullptr;
+    if (nrows <= kSolveKeep) {
+        if (!h->solve_ws) CK(dalloc(h, &h->solve_ws, solve_doubles(n, kSolveKeep)), "solve workspace");
+        ws = h->solve_ws;
+    } else {
+        CK(cudaMallocAsync(&ws, solve_doubles(n, nrows) * sizeof(double), st), "solve workspace");
+        sp->owned = ws;
+    }
+    sp->A = ws;
+    sp->rows = sp->A + n * n;
+    sp->diag = sp->rows + (size_t)nrows * n;
+    sp->est = sp->diag + CHOL_DIAG;
+    return MODAL_OK;
+}
+
+static void release(SolveSpace& sp, cudaStream_t st) {
+    if (!sp.owned) return;
+    cudaFreeAsync(sp.owned, st);
+    cudaStreamSynchronize(st);
+}
+
+// The error word that came back with the results of a solve (out[count]); clears it.
+static modal_status solve_error(modal_h h, double word, cudaStream_t st) {
+    const int e = (int)word;
+    if (!e) return MODAL_OK;
+    CK(cudaMemsetAsync(h->d_err + 1, 0, sizeof(int), st), "error word clear");
+    CK(cudaStreamSynchronize(st), "sync");
+    if (e & MODAL_DEVERR_NOTPD) return set_error(MODAL_ENOTPD, "zeta is not positive definite");
+    return set_error(MODAL_ETIMEOUT, "a device-side wait hit its spin limit");
+}
+
+// zeta = L L^T with the carried rows (alpha, then the betas) solved against L.
+static modal_status factor_with_rows(modal_h h, const SolveSpace& sp, const double* alpha, const double* beta, int B,
+                                     cudaStream_t st) {
+    const int n = h->n_max;
+    { STAGE(h, ST_SOLVE, st); CK(launch_zeta(*h, sp.A, true, st), "zeta"); }
+    CK(cudaMemcpyAsync(sp.rows, alpha, n * sizeof(double), cudaMemcpyHostToDevice, st), "alpha copy");
+    if (B > 0)
+        CK(cudaMemcpyAsync(sp.rows + n, beta, (size_t)B * n * sizeof(double), cudaMemcpyDeviceToDevice, st), "beta copy");
+    { STAGE(h, ST_SOLVE, st); CK(launch_cholesky(*h, sp.A, n, B + 1, sp.diag, st), "cholesky"); }
+    { STAGE(h, ST_SOLVE, st); CK(launch_estimates(*h, sp.rows, n, B, sp.est, st), "estimates"); }
+    return MODAL_OK;
+}
+
 modal_status modal_fnl_weights(modal_h h, const double* alpha, double* w, double* sigma, void* stream) {
     if (check_plan(h)) return MODAL_EINVAL;
     if (!alpha || !w) return set_error(MODAL_EINVAL, "alpha and w are required");
     if (h->n_cov < 2) return set_error(MODAL_ESTATE, "need at least 2 covariance simulations");
     cudaStream_t st = as_stream(stream);
-    const int n = h->n_max;
-    double* ws = nullptr;
-    CK(cudaMallocAsync(&ws, ((size_t)n * n + n + 1) * sizeof(double), st), "weights workspace");
-    double* A = ws;
-    double* v = ws + (size_t)n * n;
-    double* norm = v + n;
+    SolveSpace sp;
+    modal_status s = solve_space(h, 1, st, &sp);
+    if (s != MODAL_OK) return s;
     auto run = [&]() -> modal_status {
-        { STAGE(h, ST_SOLVE, st); CK(launch_zeta(*h, A, st), "zeta"); }
-        { STAGE(h, ST_SOLVE, st); CK(launch_cholesky(*h, A, n, st), "cholesky"); }
-        CK(cudaMemcpyAsync(v, alpha, n * sizeof(double), cudaMemcpyHostToDevice, st), "alpha copy");
-        modal_status es = read_device_error(h, st, h->d_err + 1);
-        if (es != MODAL_OK) return es;
-        { STAGE(h, ST_SOLVE, st); CK(launch_solve_rhs(*h, A, n, v, 1, st), "triangular solve"); }
-        { STAGE(h, ST_SOLVE, st); CK(launch_estimates(*h, v, n, 0, norm, st), "alpha norm"); }
-        { STAGE(h, ST_SOLVE, st); CK(launch_fnl_weights(*h, A, n, v, norm, w, st), "back substitution"); }
-        double nrm = 0.0;
-        CK(cudaMemcpyAsync(&nrm, norm, sizeof(double), cudaMemcpyDeviceToHost, st), "norm copy");
+        const modal_status f = factor_with_rows(h, sp, alpha, nullptr, 0, st);
+        if (f != MODAL_OK) return f;
+        { STAGE(h, ST_SOLVE, st); CK(launch_fnl_weights(*h, sp.A, h->n_max, sp.rows, sp.est, w, st), "back substitution"); }
+        double out[2] = {0.0, 0.0};
+        CK(cudaMemcpyAsync(out, sp.est, sizeof(out), cudaMemcpyDeviceToHost, st), "norm copy");
         CK(cudaStreamSynchronize(st), "weights sync");
-        if (!(nrm > 0.0)) return set_error(MODAL_ENOTPD, "alpha^T zeta^-1 alpha is not positive");
-        if (sigma) *sigma = std::sqrt(6.0 / nrm);
+        const modal_status es = solve_error(h, out[1], st);
+        if (es != MODAL_OK) return es;
+        if (!(out[0] > 0.0)) return set_error(MODAL_ENOTPD, "alpha^T zeta^-1 alpha is not positive");
+        if (sigma) *sigma = std::sqrt(6.0 / out[0]);
         return MODAL_OK;
     };
-    const modal_status s = run();
-    cudaFreeAsync(ws, st);
-    cudaStreamSynchronize(st);
+    s = run();
+    release(sp, st);
     return s;
 }
 
@@ -979,33 +1031,24 @@ modal_status modal_solve(modal_h h, const double* alpha, const double* beta, int
     if (!alpha || B < 0 || (B > 0 && (!beta || !fnl))) return set_error(MODAL_EINVAL, "bad arguments");
     if (h->n_cov < 2) return set_error(MODAL_ESTATE, "need at least 2 covariance simulations");
     cudaStream_t st = as_stream(stream);
-    const int n = h->n_max;
-    double* ws = nullptr;
-    CK(cudaMallocAsync(&ws, ((size_t)n * n + (size_t)(B + 1) * n + (B + 1)) * sizeof(double), st), "solve workspace");
-    double* A = ws;
-    double* rhs = ws + (size_t)n * n;
-    double* est = rhs + (size_t)(B + 1) * n;
-    modal_status s = MODAL_OK;
+    SolveSpace sp;
+    modal_status s = solve_space(h, B + 1, st, &sp);
+    if (s != MODAL_OK) return s;
     auto run = [&]() -> modal_status {
-        { STAGE(h, ST_SOLVE, st); CK(launch_zeta(*h, A, st), "zeta"); }
-        { STAGE(h, ST_SOLVE, st); CK(launch_cholesky(*h, A, n, st), "cholesky"); }
-        CK(cudaMemcpyAsync(rhs, alpha, n * sizeof(double), cudaMemcpyHostToDevice, st), "alpha copy");
-        if (B > 0) CK(cudaMemcpyAsync(rhs + n, beta, (size_t)B * n * sizeof(double), cudaMemcpyDeviceToDevice, st), "beta copy");
-        modal_status es = read_device_error(h, st, h->d_err + 1);
-        if (es != MODAL_OK) return es;
-        { STAGE(h, ST_SOLVE, st); CK(launch_solve_rhs(*h, A, n, rhs, B + 1, st), "triangular solve"); }
-        { STAGE(h, ST_SOLVE, st); CK(launch_estimates(*h, rhs, n, B, est, st), "estimates"); }
-        std::vector<double> out(B + 1);
-        CK(cudaMemcpyAsync(out.data(), est, (B + 1) * sizeof(double), cudaMemcpyDeviceToHost, st), "estimates copy");
+        const modal_status f = factor_with_rows(h, sp, alpha, beta, B, st);
+        if (f != MODAL_OK) return f;
+        std::vector<double> out(B + 2);
+        CK(cudaMemcpyAsync(out.data(), sp.est, (B + 2) * sizeof(double), cudaMemcpyDeviceToHost, st), "estimates copy");
         CK(cudaStreamSynchronize(st), "solve sync");
+        const modal_status es = solve_error(h, out[B + 1], st);
+        if (es != MODAL_OK) return es;
         if (!(out[0] > 0.0)) return set_error(MODAL_ENOTPD, "alpha^T zeta^-1 alpha is not positive");
         if (sigma) *sigma = std::sqrt(6.0 / out[0]);
         for (int b = 0; b < B; ++b) fnl[b] = out[1 + b];
         return MODAL_OK;
     };
     s = run();
-    cudaFreeAsync(ws, st);
-    cudaStreamSynchronize(st);
+    release(sp, st);
     return s;
 }
 
@@ -1015,10 +1058,11 @@ constexpr int kPowerMaxIters = 20000, kPowerCheck = 16;
 constexpr double kPowerTol = 1e-12;
 
 // Copies the host zeta0 into A and factors it in place (lower triangle = L0).
-static modal_status factor_zeta0(modal_h h, const double* zeta0, double* A, cudaStream_t st) {
+// diag: CHOL_DIAG doubles of workspace.
+static modal_status factor_zeta0(modal_h h, const double* zeta0, double* A, double* diag, cudaStream_t st) {
     const int n = h->n_max;
     CK(cudaMemcpyAsync(A, zeta0, (size_t)n * n * sizeof(double), cudaMemcpyHostToDevice, st), "zeta0 copy");
-    { STAGE(h, ST_SOLVE, st); CK(launch_cholesky(*h, A, n, st), "cholesky of zeta0"); }
+    { STAGE(h, ST_SOLVE, st); CK(launch_cholesky(*h, A, n, 0, diag, st), "cholesky of zeta0"); }
     modal_status es = read_device_error(h, st, h->d_err + 1);
     if (es == MODAL_ENOTPD) return set_error(MODAL_ENOTPD, "zeta0 is not positive definite");
     return es;
@@ -1031,7 +1075,7 @@ modal_status modal_bivector_fit(modal_h h, const double* zeta0, double* bt, doub
     cudaStream_t st = as_stream(stream);
     const int n = h->n_max;
     double* ws = nullptr;
-    CK(cudaMallocAsync(&ws, ((size_t)3 * n * n + 2 * (size_t)n + 2) * sizeof(double), st), "fit workspace");
+    CK(cudaMallocAsync(&ws, ((size_t)3 * n * n + 2 * (size_t)n + 2 + CHOL_DIAG) * sizeof(double), st), "fit workspace");
     double* L0 = ws;
     double* Z = L0 + (size_t)n * n;
     double* T = Z + (size_t)n * n;
@@ -1039,13 +1083,13 @@ modal_status modal_bivector_fit(modal_h h, const double* zeta0, double* bt, doub
     double* w = v + n;
     double* stat = w + n;
     auto run = [&]() -> modal_status {
-        modal_status s = factor_zeta0(h, zeta0, L0, st);
+        modal_status s = factor_zeta0(h, zeta0, L0, stat + 2, st);
         if (s != MODAL_OK) return s;
         {
             // whitened Z = L0^-1 zeta L0^-T: the rows of zeta (= its columns) are solved
             // against L0, giving (L0^-1 zeta)^T; its transpose's rows are solved again.
             STAGE(h, ST_SOLVE, st);
-            CK(launch_zeta(*h, Z, st), "zeta");
+            CK(launch_zeta(*h, Z, false, st), "zeta");
             CK(launch_solve_rhs(*h, L0, n, Z, n, st), "whitening solve");
             CK(launch_transpose(*h, n, Z, T, st), "transpose");
             CK(launch_solve_rhs(*h, L0, n, T, n, st), "whitening solve");
@@ -1089,13 +1133,13 @@ modal_status modal_solve_bivector(modal_h h, const double* zeta0, const double* 
     cudaStream_t st = as_stream(stream);
     const int n = h->n_max;
     double* ws = nullptr;
-    CK(cudaMallocAsync(&ws, ((size_t)n * n + (size_t)(B + 2) * n + (B + 1)) * sizeof(double), st), "solve workspace");
+    CK(cudaMallocAsync(&ws, ((size_t)n * n + (size_t)(B + 2) * n + (B + 1) + 1 + CHOL_DIAG) * sizeof(double), st), "solve workspace");
     double* L0 = ws;
     double* rhs = L0 + (size_t)n * n;
     double* dbt = rhs + (size_t)(B + 1) * n;
     double* est = dbt + n;
     auto run = [&]() -> modal_status {
-        modal_status s = factor_zeta0(h, zeta0, L0, st);
+        modal_status s = factor_zeta0(h, zeta0, L0, est + B + 2, st);
         if (s != MODAL_OK) return s;
         CK(cudaMemcpyAsync(rhs, alpha, n * sizeof(double), cudaMemcpyHostToDevice, st), "alpha copy");
         if (B > 0) CK(cudaMemcpyAsync(rhs + n, beta, (size_t)B * n * sizeof(double), cudaMemcpyDeviceToDevice, st), "beta copy");
@@ -1126,11 +1170,11 @@ modal_status modal_bivector_rotate(modal_h h, const double* zeta0, const double*
     cudaStream_t st = as_stream(stream);
     const int n = h->n_max;
     double* ws = nullptr;
-    CK(cudaMallocAsync(&ws, ((size_t)n * n + n) * sizeof(double), st), "rotate workspace");
+    CK(cudaMallocAsync(&ws, ((size_t)n * n + n + CHOL_DIAG) * sizeof(double), st), "rotate workspace");
     double* L0 = ws;
     double* dbt = L0 + (size_t)n * n;
     auto run = [&]() -> modal_status {
-        modal_status s = factor_zeta0(h, zeta0, L0, st);
+        modal_status s = factor_zeta0(h, zeta0, L0, dbt + n, st);
         if (s != MODAL_OK) return s;
         CK(cudaMemcpyAsync(dbt, bt, n * sizeof(double), cudaMemcpyHostToDevice, st), "bt copy");
         if (B > 0 && out != x)
@@ -1303,7 +1347,7 @@ modal_status modal_get_zeta(modal_h h, double* zeta) {
     double* d = nullptr;
     const size_t nn = (size_t)h->n_max * h->n_max;
     CK(cudaMalloc(&d, nn * sizeof(double)), "zeta workspace");
-    cudaError_t e = launch_zeta(*h, d, 0);
+    cudaError_t e = launch_zeta(*h, d, false, 0);
     if (e == cudaSuccess) e = cudaMemcpy(zeta, d, nn * sizeof(double), cudaMemcpyDeviceToHost);
     cudaFree(d);
     CK(e, "zeta");

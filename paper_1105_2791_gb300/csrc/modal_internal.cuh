@@ -237,8 +237,11 @@ cudaError_t launch_vring_correct(Plan& pl, const float* vring, int nrows, float2
 cudaError_t launch_ring_mean_float(Plan& pl, float* out, cudaStream_t st);
 // k_solve.cu
 cudaError_t launch_cov_accumulate(Plan& pl, const double* beta, int B, cudaStream_t st);
-cudaError_t launch_zeta(Plan& pl, double* zeta, cudaStream_t st);
-cudaError_t launch_cholesky(Plan& pl, double* A, int n, cudaStream_t st);
+cudaError_t launch_zeta(Plan& pl, double* zeta, bool lower, cudaStream_t st);
+// A: [n + nx][n] row-major, the lower triangle of the first n rows factored in place and the nx
+// rows below replaced by their forward substitutions; diag: CHOL_DIAG doubles of workspace
+constexpr int CHOL_DIAG = 32 * 32;
+cudaError_t launch_cholesky(Plan& pl, double* A, int n, int nx, double* diag, cudaStream_t st);
 cudaError_t launch_solve_rhs(Plan& pl, const double* Lc, int n, double* rhs, int nrhs, cudaStream_t st);
 cudaError_t launch_estimates(Plan& pl, const double* rhs, int n, int B, double* out, cudaStream_t st);
 // v = alpha' (forward-solved) -> w = L^-T alpha' / norm[0] (dev norm = |alpha'|^2)
