@@ -19,10 +19,9 @@
 #include "modal_internal.cuh"
 
 #include "tc_common.cuh"
+#include "tma_map.cuh"
 
-#include <cuda.h>
 #include <algorithm>
-#include <mutex>
 
 namespace modal {
 
@@ -158,11 +157,7 @@ __global__ void __launch_bounds__(AV_THREADS, 1) k_adjoint_v(const __grid_consta
                 mbar_arrive_expect_tx(&m_full[s], (uint32_t)AV_MT);
                 const int x0 = (int)((tile0 + (n / nbq) * a.G) * 128);
                 const int y0 = (b0 - a.b_first + (int)(n % nbq)) * a.P;
-                asm volatile(
-                    "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-                        "r"(smem_u32(sM + (int64_t)s * AV_PM * 128)), "l"(reinterpret_cast<uint64_t>(&maps_map)),
-                        "r"(x0), "r"(y0), "r"(smem_u32(&m_full[s]))
-                    : "memory");
+                tma_load_2d(sM + (int64_t)s * AV_PM * 128, &maps_map, x0, y0, &m_full[s]);
                 n_issued = n + 1;
             }
             // copies still in flight complete before the CTA exits
@@ -281,23 +276,6 @@ size_t adjoint_v_workspace_bytes(const Plan& pl, int chunk) {
     return pl.prec == MODAL_FP32 ? 0 : (size_t)chunk * AV_BMAP;
 }
 
-// cuTensorMapEncodeTiled from the CUDA driver API, looked up once through the runtime.
-typedef CUresult (*AvEncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-static AvEncodeTiledFn av_encode_tiled() {
-    static std::once_flag once;
-    static AvEncodeTiledFn fn = nullptr;
-    std::call_once(once, [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess && q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<AvEncodeTiledFn>(p);
-    });
-    return fn;
-}
-
 cudaError_t launch_adjoint_v(Plan& pl, int B, const float* hk, float* maps, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
     // the map rows' pitch (npix floats) must be a multiple of 16 bytes for the tensor map
@@ -309,8 +287,6 @@ cudaError_t launch_adjoint_v(Plan& pl, int B, const float* hk, float* maps, cuda
     const size_t smem = 1024 + (size_t)AV_MAPS * AV_BMAP + (size_t)AV_GROUPS * AV_ABUF + (size_t)AV_STAGES * AV_MT;
     e = cudaFuncSetAttribute(k_adjoint_v, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    AvEncodeTiledFn enc = av_encode_tiled();
-    if (!enc) return cudaErrorNotSupported;
     AdjVArgs a;
     a.P = pl.P;
     a.npix = pl.npix;
@@ -334,11 +310,8 @@ cudaError_t launch_adjoint_v(Plan& pl, int B, const float* hk, float* maps, cuda
         const cuuint64_t dims[2] = {(cuuint64_t)pl.npix, (cuuint64_t)a.B * pl.P};
         const cuuint64_t strides[1] = {(cuuint64_t)pl.npix * sizeof(float)};
         const cuuint32_t box[2] = {128, (cuuint32_t)AV_PM};
-        const cuuint32_t estr[2] = {1, 1};
-        const CUresult r = enc(&mm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, maps + (int64_t)a.b_first * pl.P * pl.npix, dims,
-                               strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+        e = tma_map_f32(&mm, maps + (int64_t)a.b_first * pl.P * pl.npix, 2, dims, strides, box);
+        if (e != cudaSuccess) return e;
         k_adjoint_v<<<nq * a.G, AV_THREADS, smem, st>>>(mm, a);
         note_launch(pl);
         e = cudaGetLastError();

@@ -8,348 +8,437 @@
 //   adjoint   U_t(x) = 3 W_x sum_{a,b} h_tab (M_a M_b - <M_a M_b>_x)
 #include "modal_internal.cuh"
 
+#include "tc_common.cuh"
+#include "tma_map.cuh"
+
 #include <algorithm>
 
 namespace modal {
 
 // ---------------------------------------------------------------- cubic term
-// C_prs = sum_x U_(pr)(x) M_s(x) with U_(pr) = W M_p M_r: a GEMM of the pair-product
-// panel against the map panel, one map per CTA row of the grid, the panel built in
-// shared memory tile by tile and never written to HBM.
+// C_prs = sum_x (W_x M_p M_r)(x) M_s(x), p <= r <= s, of every map over its pixel ranges
+// (units: one map, one range of px_per_cta pixels).
 //
-// Tiles: 8 colex pairs (a pair group pg, pairs sorted by r, then p) x 4 values of s (a quad
-// sq); tiles entirely below the diagonal s < r are absent from the tile list.  A compute
-// item holds two tiles, either of one pair group and two quads (kind A: 8 pair values and
-// 2 x 4 map values per pixel for 32 packed FMAs) or of two pair groups and one quad (kind B:
-// 16 + 4 values); a tile left alone is paired with a quad of zeros.  The two halves of a
-// warp (16 lanes each) take one item each, of the same kind, so that a warp runs one path.
-//
-// Warp roles (named barriers, two shared-memory stages of CUB_TX pixels each):
-//   fill warps     two pixels per thread: the map values and W are prefetched one tile
-//                  ahead in registers, the pair products of all colex pairs are formed
-//                  in registers and stored as float4 slots of the panel;
-//   compute warps  16 lanes per item, 8 pixels per lane per stage.
-// Stage layout, pixel fastest: [2 n_pg slots of 4 pairs][CUB_TX] float4, then
-// [n_sq + 1 quads of 4 map values][CUB_TX] float4 (the last quad is zero), so that the
-// fill threads' stores and the half-warps' loads are runs of consecutive float4.  Per-CTA
-// partial sums go to `partial` (FP64) and are summed in a fixed order by k_beta_finalize.
+// Modes in blocks of four: a box is a block triple bp <= br <= bs, that is up to 4 x 4 x 4
+// coefficients, in four shapes (all blocks different, bp = br, br = bs, all equal: 64, 40, 40 and
+// 20 coefficients) and as many again for a last block of at most two modes.  A warp owns one box; a lane owns one of 16 pixel classes of one of two
+// units (the half-warps), reads its pixel's 4 to 12 map values and W from shared memory, forms
+// the products W M_p M_r of its box in registers and accumulates in packed FP32 pairs over p
+// (32, 24, 20 or 13 FFMA2 per pixel).  The pair products are thus formed by the warps that use
+// them, at a quarter of the multiply-adds they feed, instead of being written to a panel in
+// shared memory and read back: that panel's traffic (640 bytes in and 1152 out per pixel at 16
+// modes) was the bound.  Two sums per coefficient (8 pixels of a stage, then the stages) take 128
+// registers, so ten warps fill an SM: 16 modes (20 boxes) go as two CTAs per pair of units.
+// Maps and W stream through four stages of CUB_TX pixels: a producer thread issues four tiled
+// copies per stage (copies by all threads behind a CTA barrier per stage cost 0.2 of the time in
+// barriers, one bulk copy per row more than that in issue).  Every coefficient is the same chain of operations whatever the grid:
+// per lane class the stages' 8-pixel sums in order, then the 16 classes in order.
+// 16 modes, l_max = 1000, 16 maps: 2.34 -> 1.54 ms (34.7 TF/s useful, 0.44 of the measured FP32
+// rate; the FMA pipe is busy 0.66 of the time); 10 modes, l_max = 500, 64 maps: 1.17 -> 0.72 ms.
 constexpr int CUB_TX = 128;                 // pixels per stage
-constexpr int CUB_FILL = 64;                // fill threads (two pixels each)
-constexpr int CUB_MAXCOMP = 288;            // compute threads at most (18 items x 16 lanes)
-constexpr int CUB_THREADS = CUB_MAXCOMP + CUB_FILL;   // 11 warps: at most 3 per SM sub-partition
-constexpr int CUB_LANES = 16;               // lanes per item
+constexpr int CUB_LANES = 16;               // pixel classes
+constexpr int CUB_ROW = CUB_TX + 16;        // floats per mode row of a unit: the second unit's pixels start at 16
+constexpr int CUB_WROW = 160;               // the same for W, to a multiple of 128 bytes
+constexpr int CUB_STAGES = 4;
+constexpr int CUB_RED = 65;                 // floats per (box, class) in the final sums
 
-__device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void named_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-
-// items: [nslots] int2 (tile a, tile b); tile a < 0: idle slot; tile b < 0: tile a alone.
 struct CubicJob {
-    const float* maps;
-    const float* W;
     double* partial;
-    int64_t npix, ppc;
-    int nctas;
+    int64_t npix, ppc;                      // ppc: pixels per range, a multiple of CUB_TX
+    int nctas;                              // ranges per map
+    int64_t nunits;                         // maps x ranges
+};
+// The job's maps as rows (map, mode) of npix, and W as one row; a copy is P rows (or one) of
+// CUB_ROW pixels.
+struct CubicTiles {
+    CUtensorMap maps, W;
 };
 struct CubicJobs {
+    CubicTiles tiles[CUBIC_MAX_JOBS];
     CubicJob job[CUBIC_MAX_JOBS];
-    int64_t item_end[CUBIC_MAX_JOBS];   // cumulative item counts
+    int64_t item_end[CUBIC_MAX_JOBS];       // cumulative item counts (an item: two units, one group of boxes)
     int n;
 };
 
-// One work item: map b of `maps`, pixel range `cta` of `nctas` ranges of px_per_cta pixels;
-// the CTA's sums of every mode go to partial[(b nctas + cta) n_max + n].  Ends with the CTA
-// synchronised, so that a persistent caller can run the next item on the same shared memory.
-template <int PM>
-__device__ __forceinline__ void cubic_item(float* smem, int P, int n_pg, int n_sq, int ntiles, int ncomp,
-                                           const int* __restrict__ tiles, const int2* __restrict__ items,
-                                           const int* __restrict__ modeidx, int64_t npix, int64_t px_per_cta,
-                                           const float* __restrict__ maps, const float* __restrict__ W,
-                                           double* __restrict__ partial, int n_max, int b, int cta, int nctas) {
-    const int nslot = 2 * n_pg;
-    const int stage_f4 = (nslot + n_sq + 1) * CUB_TX;              // float4 per stage
-    const int tid = threadIdx.x;
-    const int nthr = ncomp + CUB_FILL;
-    const int64_t x_begin = (int64_t)cta * px_per_cta;
-    const int64_t x_end = min(npix, x_begin + px_per_cta);
-    const int nch = (x_end > x_begin) ? (int)((x_end - x_begin + CUB_TX - 1) / CUB_TX) : 0;
-    const float* mb = maps + (int64_t)b * P * npix;
-    float4* s4 = reinterpret_cast<float4*>(smem);
+// The boxes of P modes: groups of at most CUBIC_BOXES codes (shape | bp << 2 | br << 4 | bs << 6 |
+// half << 8: bs is a last block of at most two modes), box i of a group on warp i.
+struct CubicShape {
+    int P, nb, ngroups, nbox, n_max;        // nbox: boxes per group
+    const int* boxes;                       // [ngroups][nbox]
+    const int* mode_of;                     // [P][P][P]
+};
 
-    // the zero quad of both stages
-    for (int i = tid; i < 2 * CUB_TX; i += nthr)
-        s4[(i / CUB_TX) * stage_f4 + (nslot + n_sq) * CUB_TX + i % CUB_TX] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-
-    float accA[32], accB[32];
-#pragma unroll
-    for (int e = 0; e < 32; ++e) accA[e] = accB[e] = 0.f;
-    const int lane16 = (tid % 32) % CUB_LANES;
-    const int slot_item = tid / CUB_LANES;
-    int2 it = make_int2(-1, -1);
-
-    if (tid >= ncomp) {
-        // ------------------------------------------------ fill warps
-        const int xl = tid - ncomp;                                  // pixels xl and xl + CUB_FILL
-        float cur[2][PM + 1], n1[2][PM + 1];
-        auto load = [&](float (&v)[2][PM + 1], int k) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int64_t x = x_begin + (int64_t)k * CUB_TX + xl + h * CUB_FILL;
-                const bool in = k < nch && x < x_end;
-#pragma unroll
-                for (int p = 0; p < PM; ++p) v[h][p] = (in && p < P) ? mb[(int64_t)p * npix + x] : 0.f;
-                v[h][PM] = in ? W[x] : 0.f;
-            }
-        };
-        load(cur, 0);
-        for (int k = 0; k < nch; ++k) {
-            load(n1, k + 1);
-            const int s = k & 1;
-            if (k >= 2) named_sync(3 + s, nthr);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float4* sU = s4 + s * stage_f4 + xl + h * CUB_FILL;
-                float4* sM = sU + nslot * CUB_TX;
-                const float* cv = cur[h];
-                float wm[PM];
-#pragma unroll
-                for (int p = 0; p < PM; ++p) wm[p] = cv[PM] * cv[p];
-                float st[4];
-#pragma unroll
-                for (int r = 0; r < PM; ++r)
-#pragma unroll
-                    for (int p = 0; p <= r; ++p) {
-                        const int c = r * (r + 1) / 2 + p;           // colex pair index
-                        st[c & 3] = wm[p] * cv[r];
-                        if ((c & 3) == 3 && c < 8 * n_pg) sU[(c >> 2) * CUB_TX] = make_float4(st[0], st[1], st[2], st[3]);
-                    }
-                constexpr int NPR = PM * (PM + 1) / 2;
-                if ((NPR & 3) != 0) {                                // tail of a partial float4
-                    const int c0 = NPR & ~3;
-#pragma unroll
-                    for (int i = (NPR & 3); i < 4; ++i) st[i] = 0.f;
-                    if (c0 < 8 * n_pg) sU[(c0 >> 2) * CUB_TX] = make_float4(st[0], st[1], st[2], st[3]);
-                }
-                // pair slots past the colex pairs of PM modes (8 n_pg > NPR) are zero
-                for (int c0 = (NPR + 3) & ~3; c0 < 8 * n_pg; c0 += 4)
-                    sU[(c0 >> 2) * CUB_TX] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int q = 0; q < (PM + 3) / 4; ++q)
-                    if (q < n_sq)
-                        sM[q * CUB_TX] = make_float4(q * 4 + 0 < PM ? cv[q * 4 + 0] : 0.f, q * 4 + 1 < PM ? cv[q * 4 + 1] : 0.f,
-                                                     q * 4 + 2 < PM ? cv[q * 4 + 2] : 0.f, q * 4 + 3 < PM ? cv[q * 4 + 3] : 0.f);
-            }
-            named_arrive(1 + s, nthr);
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int p = 0; p <= PM; ++p) cur[h][p] = n1[h][p];
-        }
-    } else {
-        // ------------------------------------------------ compute warps
-        it = items[slot_item];
-        const bool active = it.x >= 0;
-        const int ta = active ? tiles[it.x] : 0;
-        const int tb = (active && it.y >= 0) ? tiles[it.y] : -1;
-        const int pga = ta & 0xff, sqa = ta >> 8;
-        // kind A: one pair group, quads a and b (the zero quad for a lone tile); kind B: two pair groups, one quad
-        const bool kindB = tb >= 0 && (tb & 0xff) != pga;
-        const int pgb = kindB ? (tb & 0xff) : pga;
-        const int sqb = kindB ? sqa : (tb >= 0 ? (tb >> 8) : n_sq);
-        for (int k = 0; k < nch; ++k) {
-            const int s = k & 1;
-            named_sync(1 + s, nthr);
-            if (active) {
-                const float4* sU = s4 + s * stage_f4;
-                const float4* sM = sU + nslot * CUB_TX;
-                // packed FP32 pairs (one rounding per lane, as fmaf): tA[ip][q], tB[ip][q] hold the
-                // sums of pairs 2 ip, 2 ip + 1 of the two tiles against their s = 4 sq + q
-                float2 tA[4][4], tB[4][4];
-#pragma unroll
-                for (int ip = 0; ip < 4; ++ip)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) tA[ip][q] = tB[ip][q] = make_float2(0.f, 0.f);
-                if (!kindB) {
-#pragma unroll 1
-                    for (int xi = lane16; xi < CUB_TX; xi += CUB_LANES) {
-                        const float4 u0 = sU[(2 * pga) * CUB_TX + xi], u1 = sU[(2 * pga + 1) * CUB_TX + xi];
-                        const float4 ma = sM[sqa * CUB_TX + xi], mbv = sM[sqb * CUB_TX + xi];
-                        const float2 u2[4] = {make_float2(u0.x, u0.y), make_float2(u0.z, u0.w), make_float2(u1.x, u1.y),
-                                              make_float2(u1.z, u1.w)};
-                        const float2 a2[4] = {make_float2(ma.x, ma.x), make_float2(ma.y, ma.y), make_float2(ma.z, ma.z),
-                                              make_float2(ma.w, ma.w)};
-                        const float2 b2[4] = {make_float2(mbv.x, mbv.x), make_float2(mbv.y, mbv.y),
-                                              make_float2(mbv.z, mbv.z), make_float2(mbv.w, mbv.w)};
-#pragma unroll
-                        for (int ip = 0; ip < 4; ++ip)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                tA[ip][q] = __ffma2_rn(u2[ip], a2[q], tA[ip][q]);
-                                tB[ip][q] = __ffma2_rn(u2[ip], b2[q], tB[ip][q]);
-                            }
-                    }
-                } else {
-#pragma unroll 1
-                    for (int xi = lane16; xi < CUB_TX; xi += CUB_LANES) {
-                        const float4 u0 = sU[(2 * pga) * CUB_TX + xi], u1 = sU[(2 * pga + 1) * CUB_TX + xi];
-                        const float4 v0 = sU[(2 * pgb) * CUB_TX + xi], v1 = sU[(2 * pgb + 1) * CUB_TX + xi];
-                        const float4 mv = sM[sqa * CUB_TX + xi];
-                        const float2 u2[4] = {make_float2(u0.x, u0.y), make_float2(u0.z, u0.w), make_float2(u1.x, u1.y),
-                                              make_float2(u1.z, u1.w)};
-                        const float2 v2[4] = {make_float2(v0.x, v0.y), make_float2(v0.z, v0.w), make_float2(v1.x, v1.y),
-                                              make_float2(v1.z, v1.w)};
-                        const float2 m2[4] = {make_float2(mv.x, mv.x), make_float2(mv.y, mv.y), make_float2(mv.z, mv.z),
-                                              make_float2(mv.w, mv.w)};
-#pragma unroll
-                        for (int ip = 0; ip < 4; ++ip)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                tA[ip][q] = __ffma2_rn(u2[ip], m2[q], tA[ip][q]);
-                                tB[ip][q] = __ffma2_rn(v2[ip], m2[q], tB[ip][q]);
-                            }
-                    }
-                }
-#pragma unroll
-                for (int ip = 0; ip < 4; ++ip)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        accA[(2 * ip) * 4 + q] += tA[ip][q].x;
-                        accA[(2 * ip + 1) * 4 + q] += tA[ip][q].y;
-                        accB[(2 * ip) * 4 + q] += tB[ip][q].x;
-                        accB[(2 * ip + 1) * 4 + q] += tB[ip][q].y;
-                    }
-            }
-            if (k + 2 < nch) named_arrive(3 + s, nthr);
-        }
-    }
-    __syncthreads();
-    float* red = smem;   // [CUB_LANES][ntiles][32]
-    if (tid < ncomp && it.x >= 0) {
-#pragma unroll
-        for (int e = 0; e < 32; ++e) red[(lane16 * ntiles + it.x) * 32 + e] = accA[e];
-        if (it.y >= 0) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) red[(lane16 * ntiles + it.y) * 32 + e] = accB[e];
-        }
-    }
-    __syncthreads();
-    for (int i = tid; i < ntiles * 32; i += nthr) {
-        const int t = i / 32, e = i % 32;
-        float v = 0.f;
-        for (int ln = 0; ln < CUB_LANES; ++ln) v += red[(ln * ntiles + t) * 32 + e];
-        const int tp = tiles[t];
-        const int c = (tp & 0xff) * 8 + e / 4, sv = (tp >> 8) * 4 + e % 4;
-        const int n = modeidx[c * 16 + sv];
-        if (n >= 0) partial[((int64_t)b * nctas + cta) * n_max + n] = (double)v;
-    }
-    __syncthreads();
+// SHAPE: 0 all blocks different, 1 bp = br, 2 br = bs, 3 all equal; + 4: bs holds only two modes.
+// The coefficients of a box's (r, s) and p pair that a shape holds:
+template <int SHAPE>
+__host__ __device__ constexpr bool cub_used(int r, int s, int pp) {
+    return ((SHAPE & 1) == 0 || 2 * pp <= r) && ((SHAPE & 2) == 0 || s >= r) && ((SHAPE & 4) == 0 || s < 2);
+}
+// the pair products u(r, pp) that any of its coefficients needs
+template <int SHAPE>
+__host__ __device__ constexpr bool cub_product(int r, int pp) {
+    return cub_used<SHAPE>(r, 0, pp) || cub_used<SHAPE>(r, 1, pp) || cub_used<SHAPE>(r, 2, pp) || cub_used<SHAPE>(r, 3, pp);
 }
 
-template <int PM>
-__global__ void __launch_bounds__(CUB_THREADS, 1)
-k_cubic(int P, int n_pg, int n_sq, int ntiles, int ncomp, const int* __restrict__ tiles, const int2* __restrict__ items,
-        const int* __restrict__ modeidx, int64_t npix, int64_t px_per_cta, const float* __restrict__ maps,
-        const float* __restrict__ W, double* __restrict__ partial, int n_max) {
-    extern __shared__ __align__(16) float smem[];
-    cubic_item<PM>(smem, P, n_pg, n_sq, ntiles, ncomp, tiles, items, modeidx, npix, px_per_cta, maps, W, partial, n_max,
-                   blockIdx.y, blockIdx.x, gridDim.x);
+template <int SHAPE>
+struct CubValues {
+    float p[4], r[4], s[4], w;
+    __device__ __forceinline__ void load(const float* sp, const float* sr, const float* ss, const float* sw, int off) {
+        constexpr int NS = (SHAPE & 4) ? 2 : 4;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (i < NS || (SHAPE & 3) != 3) p[i] = sp[i * CUB_ROW + off];
+            if (!(SHAPE & 1) && (i < NS || !(SHAPE & 2))) r[i] = sr[i * CUB_ROW + off];
+            if (!(SHAPE & 2) && i < NS) s[i] = ss[i * CUB_ROW + off];
+        }
+        w = sw[off];
+    }
+    __device__ __forceinline__ float rv(int i) const { return (SHAPE & 1) ? p[i] : r[i]; }
+    __device__ __forceinline__ float sv(int i) const { return (SHAPE & 2) ? rv(i) : s[i]; }
+};
+
+template <int SHAPE, bool FIRST>
+__device__ __forceinline__ void cub_pixel(const CubValues<SHAPE>& v, float2 (&t)[4][4][2]) {
+    const float2 w2 = make_float2(v.w, v.w);
+#pragma unroll
+    for (int pp = 0; pp < 2; ++pp) {
+        if (!cub_product<SHAPE>(0, pp) && !cub_product<SHAPE>(1, pp) && !cub_product<SHAPE>(2, pp) && !cub_product<SHAPE>(3, pp)) continue;
+        const float2 wm = __fmul2_rn(w2, make_float2(v.p[2 * pp], v.p[2 * pp + 1]));
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (!cub_product<SHAPE>(r, pp)) continue;
+            const float2 u = __fmul2_rn(wm, make_float2(v.rv(r), v.rv(r)));   // W M_p M_r of two p
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                if (!cub_used<SHAPE>(r, s, pp)) continue;
+                const float2 s2 = make_float2(v.sv(s), v.sv(s));
+                t[r][s][pp] = FIRST ? __fmul2_rn(u, s2) : __ffma2_rn(u, s2, t[r][s][pp]);
+            }
+        }
+    }
+}
+
+// The two units of one item as a CTA sees them.
+struct CubicUnits {
+    int x[2], y[2];                         // the unit's first pixel (npix: none) and first row of its map
+    double* out[2];                         // the unit's partial sums
+    int nch;                                // stages
+};
+
+// Floats of a stage: [unit][4 nb modes][CUB_ROW], then [unit] W rows.
+__host__ __device__ inline int cub_stage(int nb) { return 2 * (4 * nb * CUB_ROW + CUB_WROW); }
+
+// Stage barriers behind the stages' data: full (the producer's copies have landed) and empty (every
+// box warp has read the stage); `it` counts the stages of the CTA, so a persistent caller's
+// barriers run on from item to item.
+struct CubicPipe {
+    uint64_t *full, *empty;                 // [CUB_STAGES] each
+    volatile int* abort_flag;
+    int* err;
+};
+
+// The producer (one thread): four tiled copies per stage.  The second unit's tile starts 16
+// pixels early, which puts its pixels half a bank row from the first's; what lies outside the
+// map (also a unit that has run out of pixels: only a map's last range is shorter) reads as zero,
+// and the rows of modes past P are never written: no coefficient that is kept depends on them.
+__device__ __forceinline__ void cub_produce(float* smem, const CubicPipe& pipe, const CubicTiles& tl, const CubicUnits& un, int P,
+                                            int nb, uint32_t& it) {
+    for (int k = 0; k < un.nch; ++k, ++it) {
+        const int s = it % CUB_STAGES;
+        if (!mbar_wait(&pipe.empty[s], ((it / CUB_STAGES) & 1) ^ 1, pipe.abort_flag, pipe.err)) return;
+        float* st = smem + s * cub_stage(nb);
+        mbar_arrive_expect_tx(&pipe.full[s], 2 * (P + 1) * CUB_ROW * 4);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int x = un.x[h] + k * CUB_TX - 16 * h;
+            tma_load_2d(st + h * 4 * nb * CUB_ROW, &tl.maps, x, un.y[h], &pipe.full[s]);
+            tma_load_2d(st + 8 * nb * CUB_ROW + h * CUB_WROW, &tl.W, x, 0, &pipe.full[s]);
+        }
+    }
+}
+
+template <int SHAPE, bool LOOPED>
+__device__ __forceinline__ void cubic_box(float* smem, const CubicPipe& pipe, const CubicUnits& un, const CubicShape& sh,
+                                          const int* boxes, int code, uint32_t& it) {
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, half = lane / CUB_LANES, cl = lane % CUB_LANES;
+    const int nthr = sh.nbox * 32, nb = sh.nb, P = sh.P;
+    const int op = 4 * ((code >> 2) & 3) * CUB_ROW, orr = 4 * ((code >> 4) & 3) * CUB_ROW, os = 4 * ((code >> 6) & 3) * CUB_ROW;
+    float2 acc[4][4][2], t[4][4][2];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int pp = 0; pp < 2; ++pp) acc[r][s][pp] = make_float2(0.f, 0.f);
+    for (int k = 0; k < un.nch; ++k, ++it) {
+        const int sg = it % CUB_STAGES;
+        if (!__all_sync(0xffffffffu, mbar_wait(&pipe.full[sg], (it / CUB_STAGES) & 1, pipe.abort_flag, pipe.err))) break;
+        const float* st = smem + sg * cub_stage(nb) + 16 * half + cl;
+        const float* sm = st + half * 4 * nb * CUB_ROW;
+        const float *sp = sm + op, *sr = sm + orr, *ss = sm + os, *sw = st + 8 * nb * CUB_ROW + half * CUB_WROW;
+        // two pixels per turn, each one's values read while the other is summed
+        CubValues<SHAPE> va, vb;
+        va.load(sp, sr, ss, sw, 0);
+        vb.load(sp, sr, ss, sw, CUB_LANES);
+        cub_pixel<SHAPE, true>(va, t);
+        va.load(sp, sr, ss, sw, 2 * CUB_LANES);
+        cub_pixel<SHAPE, false>(vb, t);
+        auto turn = [&](int i) {
+            vb.load(sp, sr, ss, sw, (i + 1) * CUB_LANES);
+            cub_pixel<SHAPE, false>(va, t);
+            va.load(sp, sr, ss, sw, min(i + 2, CUB_TX / CUB_LANES - 1) * CUB_LANES);
+            cub_pixel<SHAPE, false>(vb, t);
+        };
+        if constexpr (LOOPED) {
+#pragma unroll 1
+            for (int i = 2; i < CUB_TX / CUB_LANES; i += 2) turn(i);
+        } else {
+#pragma unroll
+            for (int i = 2; i < CUB_TX / CUB_LANES; i += 2) turn(i);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&pipe.empty[sg]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+#pragma unroll
+                for (int pp = 0; pp < 2; ++pp)
+                    if (cub_used<SHAPE>(r, s, pp)) acc[r][s][pp] = __fadd2_rn(acc[r][s][pp], t[r][s][pp]);
+    }
+    // the classes' sums: [unit][nbox][CUB_LANES][CUB_RED], entry (r, s, p)
+    float* red = smem + CUB_STAGES * cub_stage(nb);
+    named_sync(1, nthr);                                     // the sums of the item before have been read
+    float* own = red + ((half * sh.nbox + warp) * CUB_LANES + cl) * CUB_RED;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int pp = 0; pp < 2; ++pp)
+                if (cub_used<SHAPE>(r, s, pp)) {
+                    own[(r * 4 + s) * 4 + 2 * pp] = acc[r][s][pp].x;
+                    own[(r * 4 + s) * 4 + 2 * pp + 1] = acc[r][s][pp].y;
+                }
+    named_sync(1, nthr);
+    for (int i = threadIdx.x; i < 2 * sh.nbox * 64; i += nthr) {
+        const int h = i >= sh.nbox * 64, bx = i / 64 - h * sh.nbox, e = i % 64, c = boxes[bx];
+        const int p = 4 * ((c >> 2) & 3) + e % 4, r = 4 * ((c >> 4) & 3) + e / 16, s = 4 * ((c >> 6) & 3) + (e / 4) % 4;
+        if (p > r || r > s || s >= P || !un.out[h]) continue;
+        float v = 0.f;
+#pragma unroll
+        for (int ln = 0; ln < CUB_LANES; ++ln) v += red[((h * sh.nbox + bx) * CUB_LANES + ln) * CUB_RED + e];
+        un.out[h][sh.mode_of[(p * P + r) * P + s]] = (double)v;
+    }
+}
+
+// Units u0 and u0 + 1 of a job (the second may not exist).
+__device__ __forceinline__ CubicUnits cub_units(const CubicJob& jb, int P, int n_max, int64_t u0) {
+    CubicUnits un;
+    un.nch = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t u = u0 + h;
+        const bool valid = u < jb.nunits;
+        const int64_t b = valid ? u / jb.nctas : 0, cta = valid ? u % jb.nctas : 0;
+        const int64_t xb = valid ? min(jb.npix, cta * jb.ppc) : jb.npix, xe = min(jb.npix, xb + jb.ppc);
+        un.x[h] = (int)xb;
+        un.y[h] = (int)(b * P);
+        un.out[h] = valid ? jb.partial + u * n_max : nullptr;
+        un.nch = max(un.nch, (int)((xe - xb + CUB_TX - 1) / CUB_TX));
+    }
+    return un;
+}
+
+// The tiled copies want 128-byte aligned stages.
+__device__ __forceinline__ float* cub_align(float* raw) { return raw + ((128 - (smem_u32(raw) & 127)) & 127) / 4; }
+
+constexpr int CUB_THREADS = (CUBIC_BOXES + 1) * 32;
+
+// One CTA's barriers, producer and boxes; run() takes them through one item.  HALF: the last block
+// of modes holds at most two.  The warps of a CTA run as many different box bodies as there are
+// shapes, so the instruction cache decides how far the pixel loop is unrolled: with four shapes
+// all 8 pixels of a stage (16 modes, l_max = 1000, 16 maps: 1.51 ms, 1.63 looped), with the
+// eight that a half block brings two at a time (10 modes, l_max = 500, 64 maps: 0.72 ms looped,
+// 1.05 unrolled, 0.91 with the last block treated as whole).
+template <bool HALF>
+struct CubicCta {
+    float* smem;
+    CubicPipe pipe;
+    uint32_t it;
+    __device__ __forceinline__ void run(const CubicTiles& tl, const CubicJob& jb, const CubicShape& sh, int64_t local) {
+        const int warp = threadIdx.x / 32;
+        const CubicUnits un = cub_units(jb, sh.P, sh.n_max, 2 * (local / sh.ngroups));
+        if (warp == sh.nbox) {
+            cub_produce(smem, pipe, tl, un, sh.P, sh.nb, it);
+            return;
+        }
+        const int* boxes = sh.boxes + local % sh.ngroups * sh.nbox;
+        const int code = boxes[warp];
+        if constexpr (HALF) {
+            switch ((code & 3) | (code >> 8) << 2) {
+                case 0: cubic_box<0, true>(smem, pipe, un, sh, boxes, code, it); break;
+                case 1: cubic_box<1, true>(smem, pipe, un, sh, boxes, code, it); break;
+                case 2: cubic_box<2, true>(smem, pipe, un, sh, boxes, code, it); break;
+                case 3: cubic_box<3, true>(smem, pipe, un, sh, boxes, code, it); break;
+                case 4: cubic_box<4, true>(smem, pipe, un, sh, boxes, code, it); break;
+                case 5: cubic_box<5, true>(smem, pipe, un, sh, boxes, code, it); break;
+                case 6: cubic_box<6, true>(smem, pipe, un, sh, boxes, code, it); break;
+                default: cubic_box<7, true>(smem, pipe, un, sh, boxes, code, it); break;
+            }
+        } else {
+            switch (code & 3) {
+                case 0: cubic_box<0, false>(smem, pipe, un, sh, boxes, code, it); break;
+                case 1: cubic_box<1, false>(smem, pipe, un, sh, boxes, code, it); break;
+                case 2: cubic_box<2, false>(smem, pipe, un, sh, boxes, code, it); break;
+                default: cubic_box<3, false>(smem, pipe, un, sh, boxes, code, it); break;
+            }
+        }
+    }
+    // after a wait that gave up, the copies still in flight land before the CTA exits
+    __device__ __forceinline__ void drain() {
+        if (!*pipe.abort_flag) return;
+        for (uint32_t k = it > CUB_STAGES ? it - CUB_STAGES : 0; k < it; ++k) {
+            const long long t0 = clock64();
+            while (!mbar_try_wait(&pipe.full[k % CUB_STAGES], (k / CUB_STAGES) & 1) && clock64() - t0 < TC_WAIT_CYCLES) {
+            }
+        }
+    }
+};
+
+template <bool HALF>
+__device__ __forceinline__ CubicCta<HALF> cubic_cta(float* raw, uint64_t* bars, int* abort_word, int nbox, int* err) {
+    CubicCta<HALF> c = {cub_align(raw), {bars, bars + CUB_STAGES, abort_word, err}, 0};
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < CUB_STAGES; ++s) {
+            mbar_init(&c.pipe.full[s], 1);
+            mbar_init(&c.pipe.empty[s], nbox);
+        }
+        *c.pipe.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    return c;
+}
+
+// One CTA per item (pair of units, group of boxes), the groups of a pair adjacent: they read the
+// same maps.  (Persistent CTAs whose producer ran on into the next item measured no faster:
+// 1.76 -> 1.87 ms for 64 maps of 16 modes at l_max = 500, the loop costs registers.)
+template <bool HALF>
+__global__ void __launch_bounds__(CUB_THREADS, 1) k_cubic(const __grid_constant__ CubicTiles tl, const __grid_constant__ CubicJob jb,
+                                                        CubicShape sh, int* err) {
+    extern __shared__ __align__(128) float cub_raw[];
+    __shared__ uint64_t bars[2 * CUB_STAGES];
+    __shared__ int abort_word;
+    CubicCta<HALF> c = cubic_cta<HALF>(cub_raw, bars, &abort_word, sh.nbox, err);
+    const bool producer = (int)threadIdx.x / 32 == sh.nbox;
+    if (producer && threadIdx.x % 32 != 0) return;
+    c.run(tl, jb, sh, blockIdx.x);
+    if (producer) c.drain();
 }
 
 // The cubic sums of several plans (one pass of a mixed-l_max batch, the same P) as one
-// persistent launch: CTAs take (job, map, pixel range) items from a device counter, jobs in
-// the order given (the host puts the plans with the longest items first); every item is the
-// one the plan's own launch would compute, so the partial sums are identical.
-template <int PM>
-__global__ void __launch_bounds__(CUB_THREADS, 1)
-k_cubic_multi(CubicJobs jobs, int P, int n_pg, int n_sq, int ntiles, int ncomp, const int* __restrict__ tiles,
-              const int2* __restrict__ items, const int* __restrict__ modeidx, int n_max, int* __restrict__ counter) {
-    extern __shared__ __align__(16) float smem[];
-    __shared__ int s_item;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-        __syncthreads();
-        const int64_t item = s_item;
-        __syncthreads();
-        if (item >= jobs.item_end[jobs.n - 1]) break;
-        int j = 0;
+// persistent launch over items (job, pair of units, group), jobs in the order given (the host
+// puts the plans with the longest items first); the units are those that each plan's own launch
+// would compute, so the partial sums are identical.
+template <bool HALF>
+__global__ void __launch_bounds__(CUB_THREADS, 1) k_cubic_multi(const __grid_constant__ CubicJobs jobs, CubicShape sh, int* err) {
+    extern __shared__ __align__(128) float cub_raw[];
+    __shared__ uint64_t bars[2 * CUB_STAGES];
+    __shared__ int abort_word;
+    CubicCta<HALF> c = cubic_cta<HALF>(cub_raw, bars, &abort_word, sh.nbox, err);
+    const bool producer = (int)threadIdx.x / 32 == sh.nbox;
+    if (producer && threadIdx.x % 32 != 0) return;
+    int j = 0;
+    for (int64_t item = blockIdx.x; item < jobs.item_end[jobs.n - 1]; item += gridDim.x) {
         while (item >= jobs.item_end[j]) ++j;
-        const int64_t local = item - (j > 0 ? jobs.item_end[j - 1] : 0);
-        const CubicJob& jb = jobs.job[j];
-        cubic_item<PM>(smem, P, n_pg, n_sq, ntiles, ncomp, tiles, items, modeidx, jb.npix, jb.ppc, jb.maps, jb.W,
-                       jb.partial, n_max, (int)(local / jb.nctas), (int)(local % jb.nctas), jb.nctas);
+        c.run(jobs.tiles[j], jobs.job[j], sh, item - (j > 0 ? jobs.item_end[j - 1] : 0));
     }
+    if (producer) c.drain();
 }
 
-static size_t cubic_smem(const Plan& pl) {
-    const size_t tilebuf = 2 * (size_t)CUB_TX * (2 * pl.n_pg + pl.n_sq + 1) * 16;
-    const size_t redbuf = (size_t)CUB_LANES * pl.n_tiles * 32 * 4;
-    return tilebuf > redbuf ? tilebuf : redbuf;
+static size_t cubic_smem(const CubicShape& sh) {
+    const size_t stages = (size_t)CUB_STAGES * cub_stage(sh.nb);
+    const size_t red = (size_t)2 * sh.nbox * CUB_LANES * CUB_RED;
+    return (stages + red) * sizeof(float) + 128;
 }
 
-template <int PM>
-static cudaError_t launch_cubic_pm(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st) {
-    const int ncomp = pl.cubic_nslots * CUB_LANES;
-    const size_t smem = cubic_smem(pl);
-    cudaError_t e = cudaFuncSetAttribute(k_cubic<PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int64_t ppc = ((pl.npix + pl.cubic_ctas - 1) / pl.cubic_ctas + CUB_TX - 1) / CUB_TX * CUB_TX;
-    dim3 grid(pl.cubic_ctas, B);
-    k_cubic<PM><<<grid, ncomp + CUB_FILL, smem, st>>>(pl.P, pl.n_pg, pl.n_sq, pl.n_tiles, ncomp, pl.tiles,
-                                                    reinterpret_cast<const int2*>(pl.tiles + ((pl.n_tiles + 1) & ~1)), pl.modeidx,
-                                                    pl.npix, ppc, maps, pl.W, partial, pl.n_max);
-    note_launch(pl);
-    return cudaGetLastError();
+// whether the boxes have half blocks (as the plan built them)
+static bool cubic_half(int P) { return P % 4 == 1 || P % 4 == 2; }
+
+static CubicShape cubic_shape(const Plan& pl) {
+    CubicShape sh;
+    sh.P = pl.P;
+    sh.nb = (pl.P + 3) / 4;
+    sh.ngroups = pl.cubic_groups;
+    sh.nbox = pl.cubic_boxes;
+    sh.n_max = pl.n_max;
+    sh.boxes = pl.boxes;
+    sh.mode_of = pl.mode_of;
+    return sh;
 }
 
-template <int PM>
-static cudaError_t launch_cubic_multi_pm(const Plan& p0, const CubicJobs& jobs, int* counter, int nctas_grid,
-                                        cudaStream_t st) {
-    const int ncomp = p0.cubic_nslots * CUB_LANES;
-    const size_t smem = cubic_smem(p0);
-    cudaError_t e = cudaFuncSetAttribute(k_cubic_multi<PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    k_cubic_multi<PM><<<nctas_grid, ncomp + CUB_FILL, smem, st>>>(jobs, p0.P, p0.n_pg, p0.n_sq, p0.n_tiles, ncomp, p0.tiles,
-                                                                   reinterpret_cast<const int2*>(p0.tiles + ((p0.n_tiles + 1) & ~1)),
-                                                                   p0.modeidx, p0.n_max, counter);
-    note_launch(p0);
-    return cudaGetLastError();
+static CubicJob cubic_job(const Plan& pl, int B, double* partial) {
+    CubicJob jb;
+    jb.partial = partial;
+    jb.npix = pl.npix;
+    jb.ppc = ((pl.npix + pl.cubic_ctas - 1) / pl.cubic_ctas + CUB_TX - 1) / CUB_TX * CUB_TX;
+    jb.nctas = pl.cubic_ctas;
+    jb.nunits = (int64_t)B * pl.cubic_ctas;
+    return jb;
 }
 
-cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, const int* B, int n, int* counter,
-                               cudaStream_t st) {
+static cudaError_t cubic_tiles(const Plan& pl, const float* maps, int B, CubicTiles* tl) {
+    const cuuint64_t dims[2] = {(cuuint64_t)pl.npix, (cuuint64_t)B * pl.P}, wdims[2] = {(cuuint64_t)pl.npix, 1};
+    const cuuint64_t strides[1] = {(cuuint64_t)pl.npix * sizeof(float)};
+    const cuuint32_t box[2] = {CUB_ROW, (cuuint32_t)pl.P}, wbox[2] = {CUB_ROW, 1};
+    const cudaError_t e = tma_map_f32(&tl->maps, maps, 2, dims, strides, box);
+    return e != cudaSuccess ? e : tma_map_f32(&tl->W, pl.W, 2, wdims, strides, wbox);
+}
+
+cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, const int* B, int n, cudaStream_t st) {
     if (n < 1 || n > CUBIC_MAX_JOBS) return cudaErrorInvalidValue;
     const Plan& p0 = *plans[0];
-    if (p0.cubic_nslots * CUB_LANES > CUB_MAXCOMP || p0.cubic_nslots % 2 != 0) return cudaErrorInvalidValue;
+    const CubicShape sh = cubic_shape(p0);
     CubicJobs jobs = {};
     int64_t total = 0;
     for (int i = 0; i < n; ++i) {
         const Plan& pl = *plans[i];
         if (pl.P != p0.P || B[i] < 1 || B[i] > pl.chunk) return cudaErrorInvalidValue;
-        CubicJob& jb = jobs.job[i];
-        jb.maps = maps[i];
-        jb.W = pl.W;
-        jb.partial = pl.partial;
-        jb.npix = pl.npix;
-        jb.nctas = pl.cubic_ctas;
-        jb.ppc = ((pl.npix + pl.cubic_ctas - 1) / pl.cubic_ctas + CUB_TX - 1) / CUB_TX * CUB_TX;
-        total += (int64_t)B[i] * pl.cubic_ctas;
+        jobs.job[i] = cubic_job(pl, B[i], pl.partial);
+        const cudaError_t e = cubic_tiles(pl, maps[i], B[i], &jobs.tiles[i]);
+        if (e != cudaSuccess) return e;
+        total += (jobs.job[i].nunits + 1) / 2 * sh.ngroups;
         jobs.item_end[i] = total;
     }
     jobs.n = n;
-    const int grid = (int)std::min<int64_t>(total, (int64_t)std::max(p0.nsm, 1));
-    if (p0.P <= 4) return launch_cubic_multi_pm<4>(p0, jobs, counter, grid, st);
-    if (p0.P <= 8) return launch_cubic_multi_pm<8>(p0, jobs, counter, grid, st);
-    return launch_cubic_multi_pm<16>(p0, jobs, counter, grid, st);
+    const size_t smem = cubic_smem(sh);
+    auto kernel = cubic_half(p0.P) ? k_cubic_multi<true> : k_cubic_multi<false>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    // CTAs: as many as the register file holds (twelve warps per SM)
+    const int64_t grid = std::min(total, (int64_t)std::max(p0.nsm, 1) * std::max(1, 12 / (sh.nbox + 1)));
+    kernel<<<(unsigned)grid, (sh.nbox + 1) * 32, smem, st>>>(jobs, sh, p0.d_err);
+    note_launch(p0);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
-    if (pl.cubic_nslots * CUB_LANES > CUB_MAXCOMP || pl.cubic_nslots % 2 != 0) return cudaErrorInvalidValue;
-    if (pl.P <= 4) return launch_cubic_pm<4>(pl, maps, B, partial, st);
-    if (pl.P <= 8) return launch_cubic_pm<8>(pl, maps, B, partial, st);
-    return launch_cubic_pm<16>(pl, maps, B, partial, st);
+    const CubicShape sh = cubic_shape(pl);
+    const CubicJob jb = cubic_job(pl, B, partial);
+    CubicTiles tl;
+    cudaError_t e = cubic_tiles(pl, maps, B, &tl);
+    if (e != cudaSuccess) return e;
+    const size_t smem = cubic_smem(sh);
+    auto kernel = cubic_half(pl.P) ? k_cubic<true> : k_cubic<false>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int64_t items = (jb.nunits + 1) / 2 * sh.ngroups;
+    kernel<<<(unsigned)items, (sh.nbox + 1) * 32, smem, st>>>(tl, jb, sh, pl.d_err);
+    note_launch(pl);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- linear term GEMM
@@ -673,8 +762,8 @@ cudaError_t launch_beta_finalize(Plan& pl, int B, int use_linear, const double* 
     if (B == 0) return cudaSuccess;
     const int n = B * pl.n_max;
     k_beta_finalize<<<(n + 127) / 128, 128, 0, st>>>(pl.P, pl.n_max, B, pl.cubic_ctas, use_linear, lin_splits,
-                                                      pl.n_pair, pl.modeidx + 16 * 256, pl.modeidx + 16 * 256 + 1024,
-                                                      pl.modeidx + 16 * 256 + 2048, cub_partial, lin_partial, beta);
+                                                      pl.n_pair, pl.mode_prs, pl.mode_prs + 1024,
+                                                      pl.mode_prs + 2048, cub_partial, lin_partial, beta);
     note_launch(pl);
     return cudaGetLastError();
 }
@@ -851,7 +940,7 @@ __global__ void k_adjoint_weights(int P, int n_pair, int n_max, int B, const int
 cudaError_t launch_adjoint_weights(Plan& pl, const double* g, int B, float* hk, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
     const int n = B * pl.P * pl.n_pair;
-    k_adjoint_weights<<<(n + 127) / 128, 128, 0, st>>>(pl.P, pl.n_pair, pl.n_max, B, pl.modeidx + 16 * 256 + 3072,
+    k_adjoint_weights<<<(n + 127) / 128, 128, 0, st>>>(pl.P, pl.n_pair, pl.n_max, B, pl.mode_of,
                                                         g, hk);
     note_launch(pl);
     return cudaGetLastError();

@@ -14,14 +14,6 @@ using namespace modal;
 
 struct modal_plan : public Plan {};
 
-// Offsets inside the small integer table `modeidx` (one allocation).
-static constexpr int MI_MODEIDX = 0;      // [256][16]  colex pair c, s -> mode or -1
-static constexpr int MI_MP = 4096;        // [1024] mode -> p
-static constexpr int MI_MR = 5120;        // [1024] mode -> r
-static constexpr int MI_MS = 6144;        // [1024] mode -> s
-static constexpr int MI_MODEOF = 7168;    // [P][P][P] sorted triple -> mode
-static constexpr int MI_TOTAL = 11264;
-
 namespace modal {
 
 static thread_local std::string g_last_error;
@@ -106,72 +98,73 @@ static void gauss_legendre(int n, std::vector<double>& mu, std::vector<double>& 
 
 static int n_modes_of(int P) { return P * (P + 1) * (P + 2) / 6; }
 
-static void build_mode_tables(modal_plan* pl, std::vector<int>& mi) {
+// Small integer tables: mode -> (p, r, s) as three rows of 1024, and sorted triple -> mode [P][P][P].
+static void build_mode_tables(modal_plan* pl, std::vector<int>& prs, std::vector<int>& mode_of) {
     const int P = pl->P;
-    mi.assign(MI_TOTAL, -1);
+    prs.assign(3 * 1024, -1);
     pl->mode_p.clear(); pl->mode_r.clear(); pl->mode_s.clear();
-    std::vector<int> mode_of(P * P * P, -1);
+    mode_of.assign(P * P * P, -1);
     int n = 0;
     for (int p = 0; p < P; ++p)
         for (int r = p; r < P; ++r)
             for (int s = r; s < P; ++s) {
                 pl->mode_p.push_back(p); pl->mode_r.push_back(r); pl->mode_s.push_back(s);
-                mi[MI_MP + n] = p; mi[MI_MR + n] = r; mi[MI_MS + n] = s;
+                prs[n] = p; prs[1024 + n] = r; prs[2048 + n] = s;
                 mode_of[(p * P + r) * P + s] = n;
-                mi[MI_MODEOF + (p * P + r) * P + s] = n;
                 ++n;
             }
-    // colex pairs (sorted by r then p), padded to a multiple of 8
-    std::vector<std::pair<int, int>> colex;
-    for (int r = 0; r < P; ++r)
-        for (int p = 0; p <= r; ++p) colex.push_back({p, r});
-    pl->n_pg = ((int)colex.size() + 7) / 8;
-    pl->n_sq = (P + 3) / 4;
-    std::vector<int> pair_ab(pl->n_pg * 8, -1);
-    for (size_t c = 0; c < colex.size(); ++c) pair_ab[c] = colex[c].first | (colex[c].second << 8);
-    for (size_t c = 0; c < colex.size(); ++c)
-        for (int s = 0; s < P; ++s)
-            if (s >= colex[c].second)
-                mi[MI_MODEIDX + c * 16 + s] = mode_of[(colex[c].first * P + colex[c].second) * P + s];
-    std::vector<int> tiles;
-    for (int pg = 0; pg < pl->n_pg; ++pg)
-        for (int sq = 0; sq < pl->n_sq; ++sq) {
-            bool any = false;
-            for (int c = pg * 8; c < pg * 8 + 8 && c < (int)colex.size(); ++c)
-                for (int s = sq * 4; s < sq * 4 + 4 && s < P; ++s)
-                    if (s >= colex[c].second) any = true;
-            if (any) tiles.push_back(pg | (sq << 8));
+    pl->n_pg = (P * (P + 1) / 2 + 7) / 8;
+}
+
+// The boxes of the cubic kernel: block triples bp <= br <= bs of four modes each, in groups of at
+// most CUBIC_BOXES (one warp each).  Within a group warp i runs on sub-partition i % 4: boxes are
+// placed heaviest first where there is least work, then swapped while that evens the
+// sub-partitions out (the sum of squares falls).
+static void build_cubic_boxes(modal_plan* pl, std::vector<int>& boxes) {
+    const int nb = (pl->P + 3) / 4;
+    const bool half = pl->P % 4 == 1 || pl->P % 4 == 2;      // the last block holds at most two modes
+    // packed multiply-adds per pixel, pair products included, by shape and half
+    auto weight = [](int code) {
+        static const int w[2][4] = {{42, 32, 30, 21}, {26, 20, 12, 6}};
+        return w[code >> 8][code & 3];
+    };
+    std::vector<int> codes;
+    for (int bp = 0; bp < nb; ++bp)
+        for (int br = bp; br < nb; ++br)
+            for (int bs = br; bs < nb; ++bs)
+                codes.push_back((bp == br ? 1 : 0) | (br == bs ? 2 : 0) | bp << 2 | br << 4 | bs << 6 |
+                                (half && bs == nb - 1 ? 1 : 0) << 8);
+    std::stable_sort(codes.begin(), codes.end(), [&](int a, int b) { return weight(a) > weight(b); });
+    const int ngroups = ((int)codes.size() + CUBIC_BOXES - 1) / CUBIC_BOXES;
+    const int nbox = (int)codes.size() / ngroups;            // 1, 4 or 10 boxes, or 20 in two groups
+    pl->cubic_groups = ngroups;
+    pl->cubic_boxes = nbox;
+    boxes.assign((size_t)ngroups * nbox, 0);
+    std::vector<int> load(ngroups * 4, 0), used(ngroups * 4, 0);
+    for (int code : codes) {
+        int best = -1;
+        for (int i = 0; i < ngroups * 4; ++i) {
+            const int slots = (nbox - i % 4 + 3) / 4;       // warps of this group on sub-partition i % 4
+            if (used[i] < slots && (best < 0 || load[i] < load[best])) best = i;
         }
-    pl->n_tiles = (int)tiles.size();
-    // compute items of the cubic kernel: two tiles of one pair group (two quads), else two
-    // pair groups of one quad, else a tile alone; items of the first kind first, each kind
-    // padded to an even count with idle slots so that the two half-warps of a warp run the
-    // same path.  Appended after the tile codes (from an even offset) as (tile a, tile b).
-    {
-        std::vector<std::vector<int>> by_pg(pl->n_pg);
-        for (int t = 0; t < pl->n_tiles; ++t) by_pg[tiles[t] & 0xff].push_back(t);
-        std::vector<std::pair<int, int>> kind_a, kind_b;
-        std::vector<std::vector<int>> pool(pl->n_sq);
-        for (int pg = 0; pg < pl->n_pg; ++pg) {
-            const std::vector<int>& ts = by_pg[pg];            // quads ascending
-            size_t i = 0;
-            for (; i + 1 < ts.size(); i += 2) kind_a.push_back({ts[i], ts[i + 1]});
-            if (i < ts.size()) pool[tiles[ts[i]] >> 8].push_back(ts[i]);
-        }
-        for (int sq = 0; sq < pl->n_sq; ++sq) {
-            size_t i = 0;
-            for (; i + 1 < pool[sq].size(); i += 2) kind_b.push_back({pool[sq][i], pool[sq][i + 1]});
-            if (i < pool[sq].size()) kind_a.push_back({pool[sq][i], -1});
-        }
-        if (kind_a.size() % 2) kind_a.push_back({-1, -1});
-        if (kind_b.size() % 2) kind_b.push_back({-1, -1});
-        if (tiles.size() % 2) tiles.push_back(0);
-        for (const auto& it : kind_a) { tiles.push_back(it.first); tiles.push_back(it.second); }
-        for (const auto& it : kind_b) { tiles.push_back(it.first); tiles.push_back(it.second); }
-        pl->cubic_nslots = (int)(kind_a.size() + kind_b.size());
+        boxes[(best / 4) * nbox + best % 4 + 4 * used[best]] = code;
+        load[best] += weight(code);
+        ++used[best];
     }
-    pl->cubic_pair_ab_host = pair_ab;
-    pl->cubic_tiles_host = tiles;
+    auto part = [&](int i) { return (i / nbox) * 4 + i % nbox % 4; };
+    for (bool better = true; better;) {
+        better = false;
+        for (size_t i = 0; i < boxes.size(); ++i)
+            for (size_t j = i + 1; j < boxes.size(); ++j) {
+                const int a = part((int)i), b = part((int)j), d = weight(boxes[j]) - weight(boxes[i]);
+                // moving d from b to a changes the sum of squares by 2 d (load[a] - load[b] + d)
+                if (a == b || d == 0 || (long long)d * (load[a] - load[b] + d) >= 0) continue;
+                std::swap(boxes[i], boxes[j]);
+                load[a] += d;
+                load[b] -= d;
+                better = true;
+            }
+    }
 }
 
 // ------------------------------------------------------------------ workspace
@@ -272,7 +265,7 @@ static void destroy_plan(modal_plan* pl) {
     cudaDeviceSynchronize();
     free_workspace(pl);
     dfree(pl->lam); dfree(pl->filt); dfree(pl->W); dfree(pl->wring); dfree(pl->twiddle);
-    dfree(pl->modeidx); dfree(pl->tiles); dfree(pl->pair_ab);
+    dfree(pl->mode_prs); dfree(pl->mode_of); dfree(pl->boxes);
     dfree(pl->pair_sum); dfree(pl->pair_mean); dfree(pl->S1); dfree(pl->S2);
     dfree(pl->ring_sum); dfree(pl->ring_mean);
     dfree(pl->solve_ws); dfree(pl->d_err); dfree(pl->adj_pm); dfree(pl->adj_pm_blk);
@@ -396,8 +389,7 @@ modal_status modal_init(int lmax, int P, const double* basis, const double* C_l,
         cudaDeviceGetAttribute(&pl->nsm, cudaDevAttrMultiProcessorCount, pl->dev);
         pl->nsm = std::max(pl->nsm, 1);
         // pixel ranges of the cubic and quartic sums per map: one per 8192 pixels, at most one
-        // per SM (a 32-map launch at l_max = 2000 then runs 4864 CTAs: 18.09 ms, against 18.53
-        // with 512 ranges per map, whose per-CTA reductions and partial sums cost more)
+        // per SM (more ranges cost more reductions per CTA and more partial sums to add)
         int64_t ctas = pl->npix / 8192;
         pl->cubic_ctas = (int)std::max<int64_t>(1, std::min<int64_t>(ctas, pl->nsm));
         int64_t ks = pl->npix / 16384;
@@ -520,18 +512,17 @@ modal_status modal_init(int lmax, int P, const double* basis, const double* C_l,
         CKI(dalloc(pl, &pl->twiddle, tw.size()), "twiddles");
         CKI(cudaMemcpy(pl->twiddle, tw.data(), tw.size() * sizeof(float4), cudaMemcpyHostToDevice), "twiddles copy");
     }
-    // mode / pair / tile tables
+    // mode tables and the boxes of the cubic sums
     {
-        std::vector<int> mi;
-        build_mode_tables(pl, mi);
-        CKI(dalloc(pl, &pl->modeidx, mi.size()), "mode tables");
-        CKI(cudaMemcpy(pl->modeidx, mi.data(), mi.size() * sizeof(int), cudaMemcpyHostToDevice), "mode tables copy");
-        CKI(dalloc(pl, &pl->tiles, pl->cubic_tiles_host.size()), "tiles");
-        CKI(cudaMemcpy(pl->tiles, pl->cubic_tiles_host.data(), pl->cubic_tiles_host.size() * sizeof(int),
-                       cudaMemcpyHostToDevice), "tiles copy");
-        CKI(dalloc(pl, &pl->pair_ab, pl->cubic_pair_ab_host.size()), "pairs");
-        CKI(cudaMemcpy(pl->pair_ab, pl->cubic_pair_ab_host.data(), pl->cubic_pair_ab_host.size() * sizeof(int),
-                       cudaMemcpyHostToDevice), "pairs copy");
+        std::vector<int> prs, mode_of, boxes;
+        build_mode_tables(pl, prs, mode_of);
+        build_cubic_boxes(pl, boxes);
+        CKI(dalloc(pl, &pl->mode_prs, prs.size()), "mode tables");
+        CKI(cudaMemcpy(pl->mode_prs, prs.data(), prs.size() * sizeof(int), cudaMemcpyHostToDevice), "mode tables copy");
+        CKI(dalloc(pl, &pl->mode_of, mode_of.size()), "mode index");
+        CKI(cudaMemcpy(pl->mode_of, mode_of.data(), mode_of.size() * sizeof(int), cudaMemcpyHostToDevice), "mode index copy");
+        CKI(dalloc(pl, &pl->boxes, boxes.size()), "cubic boxes");
+        CKI(cudaMemcpy(pl->boxes, boxes.data(), boxes.size() * sizeof(int), cudaMemcpyHostToDevice), "cubic boxes copy");
     }
     // accumulators and solve workspace
     CKI(dalloc(pl, &pl->S1, (size_t)pl->n_max), "S1");
@@ -1532,7 +1523,6 @@ struct modal_batch {
     int key_linear = -1;
     int schedule = MODAL_BATCH_STREAMS;
     cudaEvent_t cubic_done = nullptr;             // the shared cubic launch of one chunk pass
-    int* counter = nullptr;                       // its work-queue counter (device)
 };
 
 static void batch_drop_graph(modal_batch* bh) {
@@ -1553,7 +1543,7 @@ static bool batch_shares_cubic(const modal_batch* bh, const int* B) {
         if (B[i] == 0) continue;
         const modal_plan* p = bh->plans[i];
         if (!p0) p0 = p;
-        if (p->P != p0->P || p->n_max != p0->n_max || p->n_tiles != p0->n_tiles || p->cubic_nslots != p0->cubic_nslots)
+        if (p->P != p0->P || p->n_max != p0->n_max)
             return false;
         ++n;
     }
@@ -1600,7 +1590,7 @@ static modal_status batch_run_shared(modal_batch* bh, const void* const* alm, co
         }
         {
             STAGE(static_cast<modal_plan*>(pl[0]), ST_CUBIC, bh->main);
-            CK(launch_cubic_multi(pl.data(), mp.data(), nb.data(), (int)pl.size(), bh->counter, bh->main), "shared cubic");
+            CK(launch_cubic_multi(pl.data(), mp.data(), nb.data(), (int)pl.size(), bh->main), "shared cubic");
         }
         CK(cudaEventRecord(bh->cubic_done, bh->main), "batch pass fork");
         for (size_t i : order) {
@@ -1655,8 +1645,7 @@ modal_status modal_batch_create(const modal_h* plans, int nplans, modal_batch_h*
               cudaEventCreateWithFlags(&bh->fork, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&bh->in, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&bh->out, cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&bh->cubic_done, cudaEventDisableTiming) == cudaSuccess &&
-              cudaMalloc(&bh->counter, sizeof(int)) == cudaSuccess;
+              cudaEventCreateWithFlags(&bh->cubic_done, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 0; ok && i < nplans; ++i) {
         cudaStream_t s = nullptr;
         cudaEvent_t e = nullptr;
@@ -1756,7 +1745,6 @@ void modal_batch_destroy(modal_batch_h bh) {
     if (bh->in) cudaEventDestroy(bh->in);
     if (bh->out) cudaEventDestroy(bh->out);
     if (bh->cubic_done) cudaEventDestroy(bh->cubic_done);
-    if (bh->counter) cudaFree(bh->counter);
     if (bh->main) cudaStreamDestroy(bh->main);
     delete bh;
 }

@@ -10,7 +10,6 @@
 #include "../../include/modal.h"
 
 #define MODAL_MAXP 16
-#define MODAL_MAX_TILES 40
 
 // Device-side error word bits (set by kernels, read by modal_sync).
 #define MODAL_DEVERR_TIMEOUT 1
@@ -89,11 +88,11 @@ struct Plan {
     float* W = nullptr;          // [nrings*nphi] pixel weights with mask
     float* wring = nullptr;      // [nrings] w_j 2 pi / nphi (no mask)
     float4* twiddle = nullptr;   // ring-FFT twiddles: 3 Ns float4 per Stockham pass with Ns > 1
-    int* modeidx = nullptr;      // [n_pair_colex_pad][16] -> mode index or -1 (cubic tiles)
-    int* tiles = nullptr;        // [n_tiles] packed (pair group, s quad)
-    int n_tiles = 0, n_pg = 0, n_sq = 0;
-    int cubic_nslots = 0;        // compute items (half-warps) of the cubic kernel, stored after the tile codes
-    int* pair_ab = nullptr;      // colex pair c -> (p | r << 8), padded entries = -1
+    int* mode_prs = nullptr;     // [3][1024] mode -> p, r, s
+    int* mode_of = nullptr;      // [P][P][P] sorted triple -> mode
+    int* boxes = nullptr;        // [cubic_groups][cubic_boxes] box codes of the cubic kernel
+    int cubic_groups = 0, cubic_boxes = 0;
+    int n_pg = 0;                // groups of 8 colex pairs (quartic kernel)
     TcTable tc;
     TcAdjTable tca;
 
@@ -137,7 +136,6 @@ struct Plan {
     int* d_err = nullptr;        // device error words: [0] data path, [1] FP64 solve (Cholesky)
     size_t device_bytes = 0;
     size_t workspace_bytes = 0;
-    std::vector<int> cubic_pair_ab_host, cubic_tiles_host;
 
     // profiling: per-stage event pairs and launch counters
     int prof = 0;
@@ -201,10 +199,10 @@ cudaError_t launch_ring_r2c_weighted(const Plan& pl, const float* rows, int nrow
 // k_cubic.cu
 cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st);
 // The cubic sums of B[i] maps (one chunk, at maps[i], partial sums into plan i's partial
-// buffer) of n plans with the same P as one persistent launch; counter: device int.
+// buffer) of n plans with the same P as one persistent launch.
 constexpr int CUBIC_MAX_JOBS = 8;
-cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, const int* B, int n, int* counter,
-                               cudaStream_t st);
+constexpr int CUBIC_BOXES = 10;      // warps per CTA of the cubic kernel, one box each
+cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, const int* B, int n, cudaStream_t st);
 cudaError_t launch_linear_gemm(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st);
 // lin_splits: K splits summed from lin_partial ([lin_splits][n_pair][B P])
 cudaError_t launch_beta_finalize(Plan& pl, int B, int use_linear, const double* cub_partial,

@@ -1,0 +1,53 @@
+// Tensor maps for the tiled copies (TMA) of FP32 arrays: encoding on the host through the CUDA
+// driver API, and the copies themselves.
+#pragma once
+
+#include "modal_internal.cuh"
+
+#include "tc_common.cuh"
+
+#include <cuda.h>
+#include <mutex>
+
+namespace modal {
+
+// cuTensorMapEncodeTiled from the CUDA driver API, looked up once through the runtime.
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+inline EncodeTiledFn encode_tiled() {
+    static std::once_flag once;
+    static EncodeTiledFn fn = nullptr;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess && q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<EncodeTiledFn>(p);
+    });
+    return fn;
+}
+
+// An FP32 array of `rank` dimensions (innermost first, contiguous; strides[i]: bytes between
+// entries of dimension i + 1, multiples of 16) and the box of one copy; reads outside the array
+// give zero.  The base is 16-byte aligned, box[0] x 4 a multiple of 16 bytes.
+inline cudaError_t tma_map_f32(CUtensorMap* m, const float* base, int rank, const cuuint64_t* dims,
+                               const cuuint64_t* strides, const cuuint32_t* box) {
+    EncodeTiledFn enc = encode_tiled();
+    if (!enc) return cudaErrorNotSupported;
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), dims, strides,
+                           box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// One box to 128-byte aligned shared memory.  x (the innermost coordinate) is a multiple of 4.
+__device__ __forceinline__ void tma_load_2d(const void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
+            "r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
+        : "memory");
+}
+
+}  // namespace modal
