@@ -26,6 +26,11 @@
 // granularity, which L2 merges.
 #include "modal_internal.cuh"
 
+#include "tc_common.cuh"
+#include "tma_map.cuh"
+
+#include <algorithm>
+
 namespace modal {
 
 constexpr int FFT_THREADS = 512;
@@ -418,6 +423,108 @@ k_ring_r2c(int L, int R, int R_half, int RH, int P, const float* __restrict__ ma
     }
 }
 
+// ---------------------------------------------------------------- synthesis, 256 <= N <= 4096
+// The same transform with the Legendre rows fetched by tiled copies.  A CTA's part of a row (m,
+// parity) is 8192 / N ring pairs, 16 bytes at N = 4096 and 64 at N = 1024, rows 8 RH bytes
+// apart: fetched by warps that is one L1 tag lookup per row piece, 4000 clocks per CTA at
+// N = 4096 beside 3000 of shared-memory work, so the copy engine brings the tile [m][ring pair]
+// of each parity instead, into the shared memory that the transform then uses.  The first pass
+// takes its inputs straight from the two tiles (element k of the spectrum from row k or,
+// conjugate, from row N - k), a thread's 16 elements being in registers before the tiles are
+// overwritten; in that pass the ring pair varies fastest over the threads, so that a warp reads
+// consecutive values.  Every value is formed by the operations of the kernel above.
+// 16 modes, us: l_max = 500, 64 maps 972 -> 760; l_max = 1000, 16 maps 1100 -> 833 (0.75 of HBM);
+// 12 maps at l_max = 2000 3.82 -> 2.85 ms.  (The analysis transform with its U~ rows written by
+// tiled copies was slower, 121 -> 178 us for 32 maps at l_max = 1000: rows of 32 bytes.)
+// Rows per copy and copies per parity; a box is a multiple of 128 bytes.
+struct FftTiles {
+    int rows, n;
+};
+static FftTiles fft_tiles(int L) {
+    const int rows = std::min(256, (L + 8) / 8 * 8);
+    return {rows, (L + rows) / rows};                        // ceil((L + 1) / rows)
+}
+
+// Transform stride: 16 / RPB past N + N / 16, so that the RPB ring pairs of half a warp fall on
+// different banks where the ring pair varies fastest.
+template <int N>
+__host__ __device__ constexpr int ft_stride() {
+    constexpr int RPB = FFT_ELEMS / N;
+    return N + N / 16 + (RPB < 16 ? 16 / RPB : 1);
+}
+
+__device__ __forceinline__ float2* ft_align(float2* raw) { return raw + ((128 - (smem_u32(raw) & 127)) & 127) / 8; }
+
+template <int LOG2N>
+__global__ void __launch_bounds__(FFT_THREADS, 2)
+k_ring_c2r_tiled(const __grid_constant__ CUtensorMap delta, FftTiles tiles, int L, int R, int R_half,
+                 const float4* __restrict__ tw, float* __restrict__ maps, int* err) {
+    constexpr int N = 1 << LOG2N;
+    constexpr int RPB = FFT_ELEMS / N;
+    constexpr int NP = ft_stride<N>();
+    constexpr int T = N / 16;
+    extern __shared__ float2 ft_raw[];
+    __shared__ uint64_t bar;
+    __shared__ int abort_flag;
+    float2* buf = ft_align(ft_raw);
+    const int mp = blockIdx.y, j0 = blockIdx.x * RPB;
+    const int ntr = min(RPB, R_half - j0);
+    const int span = tiles.n * tiles.rows * RPB;             // float2 of one parity's tile
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_arrive_expect_tx(&bar, (uint32_t)(2 * span * sizeof(float2)));
+        for (int par = 0; par < 2; ++par)
+            for (int i = 0; i < tiles.n; ++i)
+                tma_load_4d(buf + par * span + i * tiles.rows * RPB, &delta, 2 * j0, par, i * tiles.rows, mp, &bar);
+    }
+    __syncthreads();
+    const bool ok = mbar_wait(&bar, 0, &abort_flag, err);
+    if (!__syncthreads_and(ok)) {                            // gave up: let the copies land, then leave
+        if (threadIdx.x == 0) {
+            const long long t0 = clock64();
+            while (!mbar_try_wait(&bar, 0) && clock64() - t0 < TC_WAIT_CYCLES) {
+            }
+        }
+        return;
+    }
+    {
+        const int q = threadIdx.x % RPB, tl = threadIdx.x / RPB;
+        const float2 *E = buf + q, *O = E + span;
+        float2 v[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const int k = tl + r * T;
+            const int m = r < 8 ? k : N - k;
+            float2 x = make_float2(0.f, 0.f);
+            if (m <= L) {
+                const float2 e = E[m * RPB], o = O[m * RPB];
+                const float2 dn = cadd(e, o), ds = csub(e, o);
+                if (r == 0 && k == 0) x = make_float2(dn.x, ds.x);
+                else if (r < 8) x = make_float2(dn.x - ds.y, dn.y + ds.x);   // X_n + i X_s
+                else x = make_float2(dn.x + ds.y, ds.x - dn.y);              // conj(X_n) + i conj(X_s)
+            }
+            v[r] = x;
+        }
+        dft<+1, 16>(v);
+        __syncthreads();                                     // the tiles have been read
+        float2* b = buf + q * NP;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) b[17 * tl + r] = v[r];  // pad16(16 tl) + r
+    }
+    __syncthreads();
+    const int q = threadIdx.x / T, tl = threadIdx.x % T;
+    const int jn = j0 + q, js = R - 1 - jn;
+    const bool valid = q < ntr, south = valid && js != jn;
+    float* on = maps + ((int64_t)mp * R + (valid ? jn : 0)) * N;
+    float* os = maps + ((int64_t)mp * R + (south ? js : 0)) * N;
+    fft_passes_out<+1, N, 16>(buf + q * NP, tl, tw, [&](int k, float2 z) {
+        if (valid) on[k] = z.x;
+        if (south) os[k] = z.y;
+    });
+}
+
 static int ilog2(int n) {
     int r = 0;
     while ((1 << r) < n) ++r;
@@ -426,17 +533,47 @@ static int ilog2(int n) {
 
 static size_t fft_smem(int N) { return (size_t)fft_rings_per_block(N) * fft_stride(N) * sizeof(float2); }
 
+// Legendre rows [nmp][L + 1][2][RH] as an array of ring-pair columns < R_half, and the box of a CTA.
+static cudaError_t fft_rows_map(CUtensorMap* m, const Plan& pl, const float2* rows, int nmp, int rpb, const FftTiles& t) {
+    const cuuint64_t row = (cuuint64_t)pl.RH * sizeof(float2);
+    const cuuint64_t dims[4] = {2 * (cuuint64_t)pl.R_half, 2, (cuuint64_t)pl.lmax + 1, (cuuint64_t)nmp};
+    const cuuint64_t strides[3] = {row, 2 * row, 2 * row * (cuuint64_t)(pl.lmax + 1)};
+    const cuuint32_t box[4] = {2 * (cuuint32_t)rpb, 1, (cuuint32_t)t.rows, 1};
+    return tma_map_f32(m, reinterpret_cast<const float*>(rows), 4, dims, strides, box);
+}
+template <int N>
+static size_t ft_smem(const FftTiles& t) {
+    const size_t rpb = FFT_ELEMS / N, tile = 2 * (size_t)t.n * t.rows * rpb, fft = rpb * ft_stride<N>();
+    return std::max(tile, fft) * sizeof(float2) + 128;
+}
+
 template <int LOG2N>
 static cudaError_t c2r_n(const Plan& pl, const float2* delta, int nmp, float* maps, cudaStream_t st) {
     constexpr int N = 1 << LOG2N;
-    const size_t smem = fft_smem(N);
-    cudaError_t e = cudaFuncSetAttribute(k_ring_c2r<LOG2N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int RPB = fft_rings_per_block(N);
-    dim3 grid((pl.R_half + RPB - 1) / RPB, nmp);
-    k_ring_c2r<LOG2N><<<grid, FFT_THREADS, smem, st>>>(pl.lmax, pl.nrings, pl.R_half, pl.RH, delta, pl.twiddle, maps);
-    note_launch(pl);
-    return cudaGetLastError();
+    if constexpr (N >= 256 && N <= 4096) {
+        const int RPB = fft_rings_per_block(N);
+        const FftTiles t = fft_tiles(pl.lmax);
+        CUtensorMap m;
+        cudaError_t e = fft_rows_map(&m, pl, delta, nmp, RPB, t);
+        if (e != cudaSuccess) return e;
+        const size_t smem = ft_smem<N>(t);
+        e = cudaFuncSetAttribute(k_ring_c2r_tiled<LOG2N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const dim3 grid((pl.R_half + RPB - 1) / RPB, nmp);
+        k_ring_c2r_tiled<LOG2N><<<grid, FFT_THREADS, smem, st>>>(m, t, pl.lmax, pl.nrings, pl.R_half, pl.twiddle, maps, pl.d_err);
+        note_launch(pl);
+        return cudaGetLastError();
+    } else {
+        // shorter rings: a row's part is 512 bytes or more; N = 8192: 8 bytes, below a copy's 16
+        const size_t smem = fft_smem(N);
+        cudaError_t e = cudaFuncSetAttribute(k_ring_c2r<LOG2N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const int RPB = fft_rings_per_block(N);
+        dim3 grid((pl.R_half + RPB - 1) / RPB, nmp);
+        k_ring_c2r<LOG2N><<<grid, FFT_THREADS, smem, st>>>(pl.lmax, pl.nrings, pl.R_half, pl.RH, delta, pl.twiddle, maps);
+        note_launch(pl);
+        return cudaGetLastError();
+    }
 }
 
 template <int LOG2N, bool WPIX>

@@ -50,4 +50,11 @@ __device__ __forceinline__ void tma_load_2d(const void* dst, const CUtensorMap* 
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_4d(const void* dst, const CUtensorMap* map, int x, int y, int z, int w, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::
+            "r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
+        : "memory");
+}
+
 }  // namespace modal
