@@ -894,14 +894,12 @@ cudaError_t launch_pair_accumulate(Plan& pl, const float* maps, int B, cudaStrea
     if (B == 0) return cudaSuccess;
     const int64_t nblk = (pl.npix + PA_PIX - 1) / PA_PIX;
     const int grid = (int)(nblk < 152 * 16 ? nblk : 152 * 16);
-    note_launch(pl);
-    if (pl.P <= 4)
-        k_pair_accumulate<4><<<grid, PA_THREADS, pa_smem_floats<4>() * 4, st>>>(pl.P, B, pl.npix, maps, pl.pair_sum);
-    else if (pl.P <= 8)
-        k_pair_accumulate<8><<<grid, PA_THREADS, pa_smem_floats<8>() * 4, st>>>(pl.P, B, pl.npix, maps, pl.pair_sum);
-    else
-        k_pair_accumulate<16><<<grid, PA_THREADS, pa_smem_floats<16>() * 4, st>>>(pl.P, B, pl.npix, maps, pl.pair_sum);
-    return cudaGetLastError();
+    return with_even_modes(pl.P, [&](auto pm) {
+        constexpr int PM = decltype(pm)::value;
+        k_pair_accumulate<PM><<<grid, PA_THREADS, pa_smem_floats<PM>() * 4, st>>>(pl.P, B, pl.npix, maps, pl.pair_sum);
+        note_launch(pl);
+        return cudaGetLastError();
+    });
 }
 
 __global__ void k_pair_finalize(int64_t n, double inv, const double* __restrict__ sums, float* __restrict__ mean) {

@@ -195,8 +195,15 @@ k_quartic(int P, int n_pg, int n_sq, int ntiles, int nl, int ncomp, const int* _
     }
 }
 
-static int quartic_pm(int P) { return P <= 4 ? 4 : (P <= 8 ? 8 : 16); }
-static int quartic_lanes(const Plan& pl) { return std::max(1, std::min(8, QT_MAXCOMP / pl.qt.ntiles)); }
+// Modes in the panels: P rounded up to even (panels padded to 16 modes for every P > 8 gave 54 tiles
+// instead of 33 at 10 modes: quartic sums of 8 maps at l_max = 300 385 -> 255 us).
+static int quartic_pm(int P) { return (P + 1) / 2 * 2; }
+// Pixel lanes per tile, by the number of modes.  They fix the order of the FP32 sums of a CTA, so
+// they are a property of P and not of the tile list; lanes x tiles stays within QT_MAXCOMP.
+static int quartic_lanes(const Plan& pl) {
+    static const int lanes[MODAL_MAXP + 1] = {8, 8, 8, 8, 8, 8, 8, 8, 8, 7, 5, 4, 3, 2, 2, 2, 2};
+    return lanes[pl.P];
+}
 
 static size_t quartic_smem(const Plan& pl) {
     const size_t SU = 8 * (size_t)pl.n_pg + 4, SQ = 4 * (size_t)pl.qt.n_sq + 4;
@@ -223,11 +230,8 @@ static cudaError_t launch_quartic_pm(Plan& pl, const float* maps, int B, double*
 cudaError_t launch_quartic(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
     if (pl.qt.ntiles > QT_MAXCOMP) return cudaErrorInvalidValue;
-    switch (quartic_pm(pl.P)) {
-        case 4: return launch_quartic_pm<4>(pl, maps, B, partial, st);
-        case 8: return launch_quartic_pm<8>(pl, maps, B, partial, st);
-        default: return launch_quartic_pm<16>(pl, maps, B, partial, st);
-    }
+    if (pl.qt.ntiles * quartic_lanes(pl) > QT_MAXCOMP) return cudaErrorInvalidValue;
+    return with_even_modes(pl.P, [&](auto pm) { return launch_quartic_pm<decltype(pm)::value>(pl, maps, B, partial, st); });
 }
 
 // Host tables: quadruples (lexicographic), the register tiles and the map from
@@ -341,43 +345,59 @@ k_pair_ring_maps(int P, int nphi, int64_t npix, int nrings, int n_pair, const fl
     }
 }
 
-// h[b][(ab)][(cd)] = sum_j W_j <ab>_j rq[b][(cd)][j].  CTA: 8 rows (ab) x all (cd) of
-// one map; ring chunks of 32 staged in shared memory.
-constexpr int QH_ROWS = 8, QH_J = 32;
+// h[b][(ab)][(cd)] = sum_j W_j <ab>_j rq[b][(cd)][j] (scale 1, rq of map b), and the two-pair sums
+// kmat[(ab)][(cd)] = sum_j nphi W_j <ab>_j <cd>_j (scale nphi, the means themselves as rq): FP64
+// products over the rings.  An FP64 instruction takes a warp 64 clocks whatever its lanes, so the
+// lanes hold rings (every one a useful product, contiguous reads), a warp eight (cd) of one (ab),
+// and the eight partial sums are added up across the warp in nine instructions instead of
+// forty.  With 8 rows per CTA and a thread per (cd), 8 maps at l_max = 300 with 10 modes took
+// 135 us (and the two-pair sums, a thread per pair, 102), now 35 (and 18).
+constexpr int QH_CD = 8;                                     // (cd) per warp
+constexpr int QH_WARPS = 4;
 
-__global__ void __launch_bounds__(256)
-k_quartic_hring(int n_pair, int nrings, int nphi, const double* __restrict__ rq, const double* __restrict__ mean,
+__global__ void __launch_bounds__(QH_WARPS * 32)
+k_quartic_hring(int n_pair, int nrings, int nphi, double scale, const double* __restrict__ rq, const double* __restrict__ mean,
                 const float* __restrict__ W, double* __restrict__ h) {
-    __shared__ double s_rq[QH_J][137];
-    __shared__ double s_m[QH_ROWS][QH_J];
-    const int b = blockIdx.y, a0 = blockIdx.x * QH_ROWS, tid = threadIdx.x;
-    double acc[QH_ROWS];
+    const int lane = threadIdx.x % 32, ab = blockIdx.x, b = blockIdx.z;
+    const int c0 = (blockIdx.y * QH_WARPS + threadIdx.x / 32) * QH_CD;
+    if (c0 >= n_pair) return;
+    const double* m = mean + (int64_t)ab * nrings;
+    const double* r = rq + ((int64_t)b * n_pair + c0) * nrings;
+    double acc[QH_CD];
 #pragma unroll
-    for (int i = 0; i < QH_ROWS; ++i) acc[i] = 0.0;
-    const double* rb = rq + (int64_t)b * n_pair * nrings;
-    for (int j0 = 0; j0 < nrings; j0 += QH_J) {
-        for (int i = tid; i < n_pair * QH_J; i += blockDim.x) {
-            const int cd = i / QH_J, jj = i % QH_J;
-            s_rq[jj][cd] = (j0 + jj < nrings) ? rb[(int64_t)cd * nrings + j0 + jj] : 0.0;
-        }
-        for (int i = tid; i < QH_ROWS * QH_J; i += blockDim.x) {
-            const int r = i / QH_J, jj = i % QH_J;
-            const int ab = a0 + r, j = j0 + jj;
-            s_m[r][jj] = (ab < n_pair && j < nrings) ? (double)W[(int64_t)j * nphi] * mean[(int64_t)ab * nrings + j] : 0.0;
-        }
-        __syncthreads();
-        if (tid < n_pair) {
-            for (int jj = 0; jj < QH_J; ++jj) {
-                const double x = s_rq[jj][tid];
+    for (int i = 0; i < QH_CD; ++i) acc[i] = 0.0;
+    for (int j = lane; j < nrings; j += 32) {
+        double v[QH_CD];
 #pragma unroll
-                for (int r = 0; r < QH_ROWS; ++r) acc[r] = fma(s_m[r][jj], x, acc[r]);
-            }
-        }
-        __syncthreads();
+        for (int i = 0; i < QH_CD; ++i) v[i] = c0 + i < n_pair ? r[(int64_t)i * nrings + j] : 0.0;
+        const double w = (double)W[(int64_t)j * nphi] * m[j];
+#pragma unroll
+        for (int i = 0; i < QH_CD; ++i) acc[i] = fma(w, v[i], acc[i]);
     }
-    if (tid < n_pair)
-        for (int r = 0; r < QH_ROWS; ++r)
-            if (a0 + r < n_pair) h[((int64_t)b * n_pair + a0 + r) * n_pair + tid] = acc[r];
+    // halves of the eight change places with the lane 16, 8 and 4 apart, then two plain steps:
+    // lane 4 i + k (any k) ends with the sum of (cd) c0 + index(i)
+#pragma unroll
+    for (int n = QH_CD / 2, o = 16; n >= 1; n /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double send = up ? acc[i] : acc[i + n], keep = up ? acc[i + n] : acc[i];
+            acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+    // bit 16 chose the upper four, bit 8 the upper two of these, bit 4 the upper one
+    const int cd = c0 + ((lane & 16) ? 4 : 0) + ((lane & 8) ? 2 : 0) + ((lane & 4) ? 1 : 0);
+    if (lane % 4 == 0 && cd < n_pair) h[((int64_t)b * n_pair + ab) * n_pair + cd] = scale * acc[0];
+}
+
+static cudaError_t quartic_ring_products(Plan& pl, int B, double scale, const double* rq, double* out, cudaStream_t st) {
+    const int np = pl.n_pair, per = QH_CD * QH_WARPS;
+    k_quartic_hring<<<dim3(np, (np + per - 1) / per, B), QH_WARPS * 32, 0, st>>>(np, pl.nrings, pl.nphi, scale, rq, pl.ring_mean,
+                                                                               pl.W, out);
+    note_launch(pl);
+    return cudaGetLastError();
 }
 
 // Per-pixel means: out[z][(ab)][b n_pair + (cd)] = sum_{x in split z} W_x <ab>_x M_c M_d,
@@ -452,20 +472,9 @@ k_quartic_hpix(int P, int n_pair, int ncols, int64_t npix, int64_t kchunk, const
         }
 }
 
-// Two-pair term.  kmat[z][(ab)][(cd)] = sum_x W_x <ab>_x <cd>_x: per ring
-// (sum_j nphi W_j <ab>_j <cd>_j, FP64, one split) or per pixel (k_quartic_hpix against the
-// mean panel, one block per K split); then k3[q] = sum_z sum of the three pair splits.
-__global__ void k_quartic_kring(int n_pair, int nrings, int nphi, const double* __restrict__ mean,
-                                const float* __restrict__ W, double* __restrict__ kmat) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_pair * n_pair) return;
-    const int ab = i / n_pair, cd = i % n_pair;
-    double acc = 0.0;
-    for (int j = 0; j < nrings; ++j)
-        acc = fma((double)nphi * W[(int64_t)j * nphi] * mean[(int64_t)ab * nrings + j], mean[(int64_t)cd * nrings + j], acc);
-    kmat[i] = acc;
-}
-
+// Two-pair term.  kmat[z][(ab)][(cd)] = sum_x W_x <ab>_x <cd>_x: per ring (k_quartic_hring, one
+// split) or per pixel (k_quartic_hpix against the mean panel, one block per K split); then
+// k3[q] = sum_z sum of the three pair splits.
 __global__ void k_quartic_k3(int P, int n_quad, int n_pair, int nsplit, const int* __restrict__ modes,
                              const double* __restrict__ kmat, double* __restrict__ k3) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -513,24 +522,20 @@ cudaError_t launch_quartic_linear(Plan& pl, const float* maps, int B, cudaStream
     if (B == 0) return cudaSuccess;
     const int np = pl.n_pair;
     if (pl.lin_mode == MODAL_LINEAR_RING) {
-        const int PM = quartic_pm(pl.P);
-        const int npm = PM * (PM + 1) / 2;
-        const size_t smem = (size_t)npm * (QR_THREADS + 4) * sizeof(float);
-        dim3 grid(pl.nrings, B);
-        cudaError_t e;
-        if (PM == 4) {
-            k_pair_ring_maps<4><<<grid, QR_THREADS, smem, st>>>(pl.P, pl.nphi, pl.npix, pl.nrings, np, maps, pl.qt.rq);
-        } else if (PM == 8) {
-            k_pair_ring_maps<8><<<grid, QR_THREADS, smem, st>>>(pl.P, pl.nphi, pl.npix, pl.nrings, np, maps, pl.qt.rq);
-        } else {
-            if ((e = cudaFuncSetAttribute(k_pair_ring_maps<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-                return e;
-            k_pair_ring_maps<16><<<grid, QR_THREADS, smem, st>>>(pl.P, pl.nphi, pl.npix, pl.nrings, np, maps, pl.qt.rq);
-        }
-        note_launch(pl);
-        k_quartic_hring<<<dim3((np + QH_ROWS - 1) / QH_ROWS, B), 256, 0, st>>>(np, pl.nrings, pl.nphi, pl.qt.rq,
-                                                                               pl.ring_mean, pl.W, pl.qt.h);
-        note_launch(pl);
+        cudaError_t e = with_even_modes(pl.P, [&](auto pm) {
+            constexpr int PM = decltype(pm)::value;
+            constexpr size_t smem = (size_t)(PM * (PM + 1) / 2) * (QR_THREADS + 4) * sizeof(float);
+            if (smem > 48 * 1024) {
+                const cudaError_t a = cudaFuncSetAttribute(k_pair_ring_maps<PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (a != cudaSuccess) return a;
+            }
+            k_pair_ring_maps<PM><<<dim3(pl.nrings, B), QR_THREADS, smem, st>>>(pl.P, pl.nphi, pl.npix, pl.nrings, np, maps, pl.qt.rq);
+            note_launch(pl);
+            return cudaGetLastError();
+        });
+        if (e != cudaSuccess) return e;
+        e = quartic_ring_products(pl, B, 1.0, pl.qt.rq, pl.qt.h, st);
+        if (e != cudaSuccess) return e;
     } else {
         const int ncols = B * np;
         const int64_t kchunk = ((pl.npix + pl.lin_ksplit - 1) / pl.lin_ksplit + QP_TK - 1) / QP_TK * QP_TK;
@@ -546,15 +551,16 @@ cudaError_t launch_quartic_k3(Plan& pl, cudaStream_t st) {
     const int np = pl.n_pair;
     int nsplit = 1;
     if (pl.lin_mode == MODAL_LINEAR_RING) {
-        k_quartic_kring<<<(np * np + 255) / 256, 256, 0, st>>>(np, pl.nrings, pl.nphi, pl.ring_mean, pl.W, pl.qt.kmat);
+        const cudaError_t e = quartic_ring_products(pl, 1, (double)pl.nphi, pl.ring_mean, pl.qt.kmat, st);
+        if (e != cudaSuccess) return e;
     } else {
         nsplit = pl.lin_ksplit;
         const int64_t kchunk = ((pl.npix + nsplit - 1) / nsplit + QP_TK - 1) / QP_TK * QP_TK;
         dim3 grid((np + QP_TM - 1) / QP_TM, (np + QP_TN - 1) / QP_TN, nsplit);
         k_quartic_hpix<<<grid, 256, 0, st>>>(pl.P, np, np, pl.npix, kchunk, pl.pair_mean, pl.W, nullptr, nullptr,
                                              nullptr, pl.pair_mean, pl.qt.kmat);
+        note_launch(pl);
     }
-    note_launch(pl);
     k_quartic_k3<<<(pl.qt.n_quad + 255) / 256, 256, 0, st>>>(pl.P, pl.qt.n_quad, np, nsplit, pl.qt.modes, pl.qt.kmat,
                                                              pl.qt.k3);
     note_launch(pl);

@@ -68,20 +68,17 @@ k_pair_ring(int P, int B, int nphi, int64_t npix, int nrings, const float* __res
 
 cudaError_t launch_pair_ring(Plan& pl, const float* maps, int B, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
-    note_launch(pl);
-    if (pl.P <= 4) {
-        const size_t smem = 10 * (RP_THREADS + 4) * sizeof(float);
-        k_pair_ring<4><<<pl.nrings, RP_THREADS, smem, st>>>(pl.P, B, pl.nphi, pl.npix, pl.nrings, maps, pl.ring_sum);
-    } else if (pl.P <= 8) {
-        const size_t smem = 36 * (RP_THREADS + 4) * sizeof(float);
-        k_pair_ring<8><<<pl.nrings, RP_THREADS, smem, st>>>(pl.P, B, pl.nphi, pl.npix, pl.nrings, maps, pl.ring_sum);
-    } else {
-        const size_t smem = 136 * (RP_THREADS + 4) * sizeof(float);
-        cudaError_t e = cudaFuncSetAttribute(k_pair_ring<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_pair_ring<16><<<pl.nrings, RP_THREADS, smem, st>>>(pl.P, B, pl.nphi, pl.npix, pl.nrings, maps, pl.ring_sum);
-    }
-    return cudaGetLastError();
+    return with_even_modes(pl.P, [&](auto pm) {
+        constexpr int PM = decltype(pm)::value;
+        constexpr size_t smem = (size_t)(PM * (PM + 1) / 2) * (RP_THREADS + 4) * sizeof(float);
+        if (smem > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(k_pair_ring<PM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        k_pair_ring<PM><<<pl.nrings, RP_THREADS, smem, st>>>(pl.P, B, pl.nphi, pl.npix, pl.nrings, maps, pl.ring_sum);
+        note_launch(pl);
+        return cudaGetLastError();
+    });
 }
 
 __global__ void k_ring_finalize(int64_t n, double inv, const double* __restrict__ sum, double* __restrict__ mean) {

@@ -5,6 +5,7 @@
 #include <cstdint>
 #include <cstddef>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/modal.h"
@@ -16,6 +17,22 @@
 #define MODAL_DEVERR_NOTPD 2
 
 namespace modal {
+
+// Kernels that hold one value per mode in registers are compiled for every even number of modes:
+// f(std::integral_constant<int, PM>) with PM = P rounded up to even.
+template <class F>
+inline cudaError_t with_even_modes(int P, F f) {
+    switch ((P + 1) / 2) {
+        case 1: return f(std::integral_constant<int, 2>());
+        case 2: return f(std::integral_constant<int, 4>());
+        case 3: return f(std::integral_constant<int, 6>());
+        case 4: return f(std::integral_constant<int, 8>());
+        case 5: return f(std::integral_constant<int, 10>());
+        case 6: return f(std::integral_constant<int, 12>());
+        case 7: return f(std::integral_constant<int, 14>());
+        default: return f(std::integral_constant<int, 16>());
+    }
+}
 
 inline int64_t alm_index(int64_t l, int64_t m, int64_t lmax) { return m * (2 * lmax + 3 - m) / 2 + (l - m); }
 __host__ __device__ inline int64_t d_alm_index(int64_t l, int64_t m, int64_t lmax) {
