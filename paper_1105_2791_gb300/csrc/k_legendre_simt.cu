@@ -11,58 +11,94 @@
 
 namespace modal {
 
-template <int PM>
+// A thread owns one ring pair and MB maps: a value of lambda and the filter values of its l,
+// broadcast from shared memory, then serve all of them, and a row of the table is read once per
+// MB WM maps.  WM of a block's four warps lie along the maps and the others along ring pairs, so
+// that ring counts are padded to 32 where several maps fill the block.  Bound by instruction
+// issue as scalar code, so the products and sums are packed FP32 pairs over modes (two roundings
+// as before: the product lambda a, then one FMA per mode, l ascending).  us, before and after:
+// 21 maps, l_max = 250, 8 modes 189 -> 123; 16 maps, l_max = 500, 10 modes 1320 -> 734; 8 maps,
+// l_max = 1000, 16 modes 5131 -> 3728 (34 TF/s).
+template <int PM, int MB, int WM>
 __global__ void __launch_bounds__(128)
-k_legendre_simt(int L, int P, int R, int R_half, int RH, const float* __restrict__ lam,
+k_legendre_simt(int L, int P, int B, int R_half, int RH, const float* __restrict__ lam,
                 const float* __restrict__ filt, const float2* __restrict__ alm, int64_t n_alm,
                 float2* __restrict__ delta) {
-    constexpr int CH = 64;
-    __shared__ float2 sa[CH];
+    constexpr int CH = 64, NM = MB * WM, WR = 4 / WM;
+    __shared__ __align__(16) float4 sa[CH][NM];                 // (re, re, im, im): operands of packed products
     __shared__ __align__(16) float sf[CH][PM];
-    const int m = blockIdx.y, b = blockIdx.z;
-    const int j = blockIdx.x * 128 + threadIdx.x;
+    const int m = blockIdx.y, b0 = blockIdx.z * NM;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int wm = warp % WM;                                   // this warp's maps: b0 + wm MB ..
+    const int j = (blockIdx.x * WR + warp / WM) * 32 + lane;
     const int64_t base = d_alm_index(m, m, L);
-    const float2* a = alm + (int64_t)b * n_alm + base;
-    const bool active = j < R_half;
+    const bool active = j < R_half && b0 + wm * MB < B;
+    const int last = L - m;                                     // the last row of this order
     const float* lp = lam + base * (int64_t)RH + (active ? j : 0);
 
-    float2 accE[PM], accO[PM];
+    // sums of one parity: real and imaginary parts of two modes at a time
+    float2 re[2][MB][PM / 2], im[2][MB][PM / 2];
 #pragma unroll
-    for (int p = 0; p < PM; ++p) {
-        accE[p] = make_float2(0.f, 0.f);
-        accO[p] = make_float2(0.f, 0.f);
-    }
-    for (int l0 = m; l0 <= L; l0 += CH) {
-        const int n = min(CH, L + 1 - l0);
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int k = 0; k < MB; ++k)
+#pragma unroll
+            for (int p = 0; p < PM / 2; ++p) re[e][k][p] = im[e][k][p] = make_float2(0.f, 0.f);
+    // the next eight values of lambda are on their way while eight are used; rows past the last
+    // repeat it (their a_lm are zero)
+    float lv[8], ln[8];
+    auto fetch = [&](int d) {
+        if (d + 7 <= last) {
+            const float* q = lp + (int64_t)d * RH;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ln[u] = q[(int64_t)u * RH];
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ln[u] = lp[(int64_t)min(d + u, last) * RH];
+        }
+    };
+    fetch(0);
+    for (int d0 = 0; d0 <= last; d0 += CH) {
+        const int n = min(CH, last + 1 - d0);
         __syncthreads();
-        for (int i = threadIdx.x; i < CH; i += 128) sa[i] = (i < n) ? a[l0 - m + i] : make_float2(0.f, 0.f);
+        for (int i = threadIdx.x; i < CH * NM; i += 128) {
+            const int li = i % CH, k = i / CH;
+            const float2 a = (li < n && b0 + k < B) ? alm[(int64_t)(b0 + k) * n_alm + base + d0 + li] : make_float2(0.f, 0.f);
+            sa[li][k] = make_float4(a.x, a.x, a.y, a.y);
+        }
         for (int i = threadIdx.x; i < CH * PM; i += 128) {
             const int li = i / PM, p = i % PM;
-            sf[li][p] = (li < n && p < P) ? filt[(int64_t)p * (L + 1) + l0 + li] : 0.f;
+            sf[li][p] = (li < n && p < P) ? filt[(int64_t)p * (L + 1) + m + d0 + li] : 0.f;
         }
         __syncthreads();
         if (active) {
-            // l0 - m is a multiple of CH (even), so i + u has the parity of u.
+            // d0 is a multiple of CH (even), so i + u has the parity of u.
             for (int i = 0; i < n; i += 8) {
-                float lv[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) lv[u] = (i + u < n) ? lp[(int64_t)(l0 - m + i + u) * RH] : 0.f;
+                for (int u = 0; u < 8; ++u) lv[u] = ln[u];
+                fetch(d0 + i + 8);
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    const float2 t = make_float2(lv[u] * sa[i + u].x, lv[u] * sa[i + u].y);
-                    float2* acc = (u & 1) ? accO : accE;
+                    float2 tr[MB], ti[MB];
+                    const float2 l2 = make_float2(lv[u], lv[u]);
+#pragma unroll
+                    for (int k = 0; k < MB; ++k) {
+                        const float4 a = sa[i + u][wm * MB + k];
+                        tr[k] = __fmul2_rn(l2, make_float2(a.x, a.y));
+                        ti[k] = __fmul2_rn(l2, make_float2(a.z, a.w));
+                    }
                     const float4* f4 = reinterpret_cast<const float4*>(&sf[i + u][0]);
 #pragma unroll
                     for (int q = 0; q < PM / 4; ++q) {
                         const float4 f = f4[q];
-                        acc[4 * q + 0].x = fmaf(f.x, t.x, acc[4 * q + 0].x);
-                        acc[4 * q + 0].y = fmaf(f.x, t.y, acc[4 * q + 0].y);
-                        acc[4 * q + 1].x = fmaf(f.y, t.x, acc[4 * q + 1].x);
-                        acc[4 * q + 1].y = fmaf(f.y, t.y, acc[4 * q + 1].y);
-                        acc[4 * q + 2].x = fmaf(f.z, t.x, acc[4 * q + 2].x);
-                        acc[4 * q + 2].y = fmaf(f.z, t.y, acc[4 * q + 2].y);
-                        acc[4 * q + 3].x = fmaf(f.w, t.x, acc[4 * q + 3].x);
-                        acc[4 * q + 3].y = fmaf(f.w, t.y, acc[4 * q + 3].y);
+                        const float2 fv[2] = {make_float2(f.x, f.y), make_float2(f.z, f.w)};
+#pragma unroll
+                        for (int k = 0; k < MB; ++k)
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {
+                                re[u & 1][k][2 * q + c] = __ffma2_rn(fv[c], tr[k], re[u & 1][k][2 * q + c]);
+                                im[u & 1][k][2 * q + c] = __ffma2_rn(fv[c], ti[k], im[u & 1][k][2 * q + c]);
+                            }
                     }
                 }
             }
@@ -70,29 +106,51 @@ k_legendre_simt(int L, int P, int R, int R_half, int RH, const float* __restrict
     }
     if (!active) return;
 #pragma unroll
-    for (int p = 0; p < PM; ++p) {
-        if (p < P) {
-            const int64_t row = ((int64_t)(b * P + p) * (L + 1) + m) * 2 * RH;
-            delta[row + j] = accE[p];
-            delta[row + RH + j] = accO[p];
+    for (int k = 0; k < MB; ++k) {
+        const int b = b0 + wm * MB + k;
+        if (b >= B) break;
+#pragma unroll
+        for (int p = 0; p < PM; ++p) {
+            if (p < P) {
+                const int64_t row = ((int64_t)(b * P + p) * (L + 1) + m) * 2 * RH;
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    delta[row + e * RH + j] = (p & 1) ? make_float2(re[e][k][p / 2].y, im[e][k][p / 2].y)
+                                                      : make_float2(re[e][k][p / 2].x, im[e][k][p / 2].x);
+            }
         }
     }
 }
 
+template <int PM, int MB, int WM>
+static void legendre_simt_launch(const Plan& pl, const float2* alm, int B, float2* delta, cudaStream_t st) {
+    constexpr int rings = 32 * (4 / WM), maps = MB * WM;
+    const dim3 grid((pl.R_half + rings - 1) / rings, pl.lmax + 1, (B + maps - 1) / maps);
+    k_legendre_simt<PM, MB, WM><<<grid, 128, 0, st>>>(pl.lmax, pl.P, B, pl.R_half, pl.RH, pl.lam, pl.filt, alm, pl.n_alm, delta);
+    note_launch(pl);
+}
+
+template <int PM>
+static cudaError_t legendre_simt_pm(const Plan& pl, const float2* alm, int B, float2* delta, cudaStream_t st) {
+    // as many of the block's warps along the maps as there are maps for; two maps per thread where
+    // their sums leave room for three warps per sub-partition (16 modes, 16 maps, l_max = 500:
+    // 971 us with one, 1153 with two; 10 modes 861 and 734)
+    constexpr int MB = PM <= 12 ? 2 : 1;
+    if (B == 1) legendre_simt_launch<PM, 1, 1>(pl, alm, B, delta, st);
+    else if (B <= MB) legendre_simt_launch<PM, MB, 1>(pl, alm, B, delta, st);
+    else if (B <= 2 * MB) legendre_simt_launch<PM, MB, 2>(pl, alm, B, delta, st);
+    else legendre_simt_launch<PM, MB, 4>(pl, alm, B, delta, st);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_legendre_simt(const Plan& pl, const float2* alm, int B, float2* delta, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
-    dim3 grid((pl.R_half + 127) / 128, pl.lmax + 1, B);
-    note_launch(pl);
-    if (pl.P <= 4)
-        k_legendre_simt<4><<<grid, 128, 0, st>>>(pl.lmax, pl.P, pl.nrings, pl.R_half, pl.RH, pl.lam, pl.filt,
-                                                 alm, pl.n_alm, delta);
-    else if (pl.P <= 8)
-        k_legendre_simt<8><<<grid, 128, 0, st>>>(pl.lmax, pl.P, pl.nrings, pl.R_half, pl.RH, pl.lam, pl.filt,
-                                                 alm, pl.n_alm, delta);
-    else
-        k_legendre_simt<16><<<grid, 128, 0, st>>>(pl.lmax, pl.P, pl.nrings, pl.R_half, pl.RH, pl.lam, pl.filt,
-                                                  alm, pl.n_alm, delta);
-    return cudaGetLastError();
+    switch ((pl.P + 3) / 4) {
+        case 1: return legendre_simt_pm<4>(pl, alm, B, delta, st);
+        case 2: return legendre_simt_pm<8>(pl, alm, B, delta, st);
+        case 3: return legendre_simt_pm<12>(pl, alm, B, delta, st);
+        default: return legendre_simt_pm<16>(pl, alm, B, delta, st);
+    }
 }
 
 // Transposed sums:  G_{b,t,lm} = sum_j lambda_lm(theta_j) U^{par(l-m)}_{b,t,m}(j), where
