@@ -6,7 +6,7 @@
 //
 //   map part   U^M_t(x) = W_x sum_a M_a(x) V_{t,a}(x),   V_{t,a}(x) = sum_b G_t[a][b] M_b(x),
 //              G_t[a][b] = h_{t,(a,b)} for a <= b and 0 otherwise.  Per map, V is a GEMM with
-//              M = 128 pixels, N = 16 P columns (t, a), K = 16 (b, zero-padded): six tcgen05
+//              M = 128 pixels, N = 8, 12 or 16 P columns (t, a), K = 8 or 16 (b, zero-padded): up to six tcgen05
 //              MMAs per pixel tile (two K steps of 8 tf32, hi*hi + hi*lo + lo*hi) at the wide
 //              N where an MMA instruction is cheapest per flop; the epilogue forms U^M_t from
 //              V in FP32 and writes it over the maps.
@@ -26,9 +26,7 @@
 namespace modal {
 
 constexpr int AV_PM = 16;                         // b (K) and a padded to 16
-constexpr int AV_GROUPS = 2;                      // converter/epilogue groups (one TMEM accumulator each)
 constexpr int AV_GW = 8;                          // warps per group: two per TMEM lane quarter, split by t
-constexpr int AV_THREADS = 32 * (AV_GW * AV_GROUPS + 2);   // groups, the loader warp, the MMA warp
 constexpr int AV_MAPS = 4;                        // maps per CTA (their G operands stay in shared memory)
 constexpr int AV_ROW = 64;                        // bytes of K per operand row (16 tf32)
 constexpr int AV_SBO = 8 * AV_ROW;                // bytes between 8-row groups (512 = TC_SBO)
@@ -61,19 +59,48 @@ __device__ __forceinline__ void av_ld32(uint32_t c, uint32_t (&r)[32]) {
     asm volatile(AV_LD16 : AV_R16(16) : "r"(c + 16));
     asm volatile("tcgen05.wait::ld.sync.aligned;" : AV_W16(0), AV_W16(16) :: "memory");
 }
+#define AV_R8(o) "=r"(r[o + 0]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), \
+    "=r"(r[o + 6]), "=r"(r[o + 7])
+#define AV_W8(o) "+r"(r[o + 0]), "+r"(r[o + 1]), "+r"(r[o + 2]), "+r"(r[o + 3]), "+r"(r[o + 4]), "+r"(r[o + 5]), \
+    "+r"(r[o + 6]), "+r"(r[o + 7])
+__device__ __forceinline__ void av_ld24(uint32_t c, uint32_t (&r)[32]) {
+    asm volatile(AV_LD16 : AV_R16(0) : "r"(c));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : AV_R8(16) : "r"(c + 16));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : AV_W16(0), AV_W8(16) :: "memory");
+}
 #undef AV_R16
 #undef AV_W16
+#undef AV_R8
+#undef AV_W8
 #undef AV_LD16
+
+// Columns per t: P rounded up to 8, 12 or 16 (of which a < P are used), the t read per wait and
+// the MMA's N.
+constexpr int av_cols(int P) { return P <= 8 ? 8 : (P <= 12 ? 12 : 16); }
+template <int AC>
+struct AvShape {
+    static constexpr int TT = AC == 8 ? 4 : 2;               // t per TMEM wait (32, 24 or 32 columns)
+    static constexpr int KS = AC == 8 ? 1 : 2;               // K steps of 8 tf32
+    // converter/epilogue groups, one TMEM accumulator of COLS columns each: a group spends most
+    // of a tile-map waiting (its operand's MMAs, its accumulator's reads), so three run where
+    // the accumulators fit 512 columns.  500 x 1024 grid, 16 maps, 12 modes: 505 us with two
+    // groups of 16 columns per t and t split 8 + 4, 463 with 12 columns and 6 + 6,
+    // 377 with three groups; 8 modes 451 -> 282.
+    static constexpr int GROUPS = AC == 16 ? 2 : 3;
+    static constexpr int COLS = AC == 16 ? 256 : 160;
+    static constexpr int THREADS = 32 * (AV_GW * GROUPS + 2); // groups, the loader warp, the MMA warp
+    __host__ __device__ static int n(int P) { return (AC * P + 15) / 16 * 16; }
+};
 
 // Byte offset of element (row r, k) in a K-major no-swizzle operand tile of AV_ROW bytes per row.
 __host__ __device__ constexpr int av_off(int r, int k) { return (r / 8) * AV_SBO + (k / 4) * 128 + (r % 8) * 16 + (k % 4) * 4; }
 
-// G operands: [map][hi tile, lo tile]; row n = 16 t + a, column k = b.
-__global__ void __launch_bounds__(256) k_adjv_gprep(int P, int n_pair, const float* __restrict__ hk, char* __restrict__ out) {
+// G operands: [map][hi tile, lo tile]; row n = AC t + a, column k = b.
+__global__ void __launch_bounds__(256) k_adjv_gprep(int P, int AC, int n_pair, const float* __restrict__ hk, char* __restrict__ out) {
     const int bmap = blockIdx.x;
     char* dst = out + (int64_t)bmap * AV_BMAP;
     for (int e = threadIdx.x; e < 256 * AV_PM; e += blockDim.x) {
-        const int n = e / AV_PM, k = e % AV_PM, t = n / AV_PM, a = n % AV_PM;
+        const int n = e / AV_PM, k = e % AV_PM, t = n / AC, a = n % AC;
         float v = 0.f;
         if (t < P && a < P && k < P && a <= k) {
             const int c = a * P - a * (a - 1) / 2 + (k - a);
@@ -97,13 +124,15 @@ struct AdjVArgs {
 
 // grid: n_quads * G CTAs; CTA (quad q, column c) keeps maps b_first + 4 q .. + 3 and walks
 // pixel tiles c, c + G, ...; its tile-maps n = (tile index) * nbq + (map of the quad) are
-// dealt to the two groups alternately.  One thread of its own warp issues every MMA (its
+// dealt to the groups in turn.  One thread of its own warp issues every MMA (its
 // warp-mates wait at the final barrier: a lane spinning on an mbarrier in the issuer's warp
 // would hold each issue back).  The loader warp streams each tile-map's 16 x 128
 // map values into a ring of AV_STAGES shared-memory tiles by 2D TMA (maps_map: rows b P + p
 // of the chunk's maps, boxes of 128 pixels x 16 rows; rows and pixels past the end read as
 // zero), so that several tiles per SM are in flight.
-__global__ void __launch_bounds__(AV_THREADS, 1) k_adjoint_v(const __grid_constant__ CUtensorMap maps_map, AdjVArgs a) {
+template <int AC>
+__global__ void __launch_bounds__(AvShape<AC>::THREADS, 1) k_adjoint_v(const __grid_constant__ CUtensorMap maps_map, AdjVArgs a) {
+    constexpr int AV_GROUPS = AvShape<AC>::GROUPS;
     extern __shared__ __align__(1024) char av_smem[];
     char* sG = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(av_smem) + 1023) & ~uintptr_t(1023));
     char* sA = sG + AV_MAPS * AV_BMAP;             // [AV_GROUPS][hi, lo]
@@ -172,9 +201,9 @@ __global__ void __launch_bounds__(AV_THREADS, 1) k_adjoint_v(const __grid_consta
             }
         }
     } else if (warp == AV_GW * AV_GROUPS + 1) {
-        // ---------------- MMA issuer: tile-map n goes to group n % 2's accumulator
+        // ---------------- MMA issuer: tile-map n goes to group n % GROUPS's accumulator
         if (lane == 0 && n_tm > 0) {
-            const uint32_t idesc = umma_idesc(2, AV_PM * a.P);
+            const uint32_t idesc = umma_idesc(2, AvShape<AC>::n(a.P));
             bool ok = mbar_wait(&gbar, 0, abort_flag, a.err);
             for (int64_t n = 0; ok && n < n_tm; ++n) {
                 const int g = (int)(n % AV_GROUPS);
@@ -182,11 +211,11 @@ __global__ void __launch_bounds__(AV_THREADS, 1) k_adjoint_v(const __grid_consta
                 ok = mbar_wait(&a_full[g], k & 1, abort_flag, a.err);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t dcol = tmem + (uint32_t)(g * 256);
+                const uint32_t dcol = tmem + (uint32_t)(g * AvShape<AC>::COLS);
                 const uint32_t aHi_s = smem_u32(sA + g * AV_ABUF), aLo_s = aHi_s + AV_AT;
                 const uint32_t gHi_s = smem_u32(sG + (int)(n % nbq) * AV_BMAP), gLo_s = gHi_s + AV_GT;
 #pragma unroll
-                for (int s = 0; s < 2; ++s) {
+                for (int s = 0; s < AvShape<AC>::KS; ++s) {
                     const uint32_t ko = (uint32_t)(s * 2 * 128);     // two core matrices = 8 tf32 of K
                     const uint64_t ah = umma_desc(aHi_s + ko), al = umma_desc(aLo_s + ko);
                     const uint64_t bh = umma_desc(gHi_s + ko), bl = umma_desc(gLo_s + ko);
@@ -198,14 +227,17 @@ __global__ void __launch_bounds__(AV_THREADS, 1) k_adjoint_v(const __grid_consta
             }
         }
     } else {
-        // ---------------- converter / epilogue groups: warp (quarter, half) converts K values
-        // 8 half .. + 7 of its pixels and forms U^M_t for t = 8 half .. + 7
+        // ---------------- converter / epilogue groups: warp (quarter, half) converts half of the K
+        // values of its pixels and forms U^M_t for half of the blocks of TT values of t
+        constexpr int TT = AvShape<AC>::TT, NKC = 2 * AvShape<AC>::KS;
         const int g = warp / AV_GW, quarter = warp % 4, half = (warp % AV_GW) / 4;
         const int xl = quarter * 32 + lane;              // pixel within the tile = TMEM lane
-        const uint32_t dcol = tmem + (uint32_t)(g * 256);
+        const uint32_t dcol = tmem + (uint32_t)(g * AvShape<AC>::COLS);
         const uint32_t lane_base = dcol + ((uint32_t)(quarter * 32) << 16);
         char* aHi = sA + g * AV_ABUF;
         char* aLo = aHi + AV_AT;
+        const int nblk = (a.P + TT - 1) / TT, mid = (nblk + 1) / 2;
+        const int t_begin = half ? mid * TT : 0, t_end = half ? a.P : min(a.P, mid * TT);
         uint32_t u = 0;                                  // tile-maps this group has handed to the MMA warp
         bool ok = true;
         for (int64_t n = g; ok && n < n_tm; n += AV_GROUPS, ++u) {
@@ -225,8 +257,8 @@ __global__ void __launch_bounds__(AV_THREADS, 1) k_adjoint_v(const __grid_consta
             if (lane == 0) mbar_arrive(&m_empty[s]);
             // A operand: this pixel's row of M (k = b), tf32 hi and lo, this half's K values
 #pragma unroll
-            for (int kc = 0; kc < AV_PM / 4; ++kc) {
-                if ((kc >> 1) != half) continue;         // (compile-time kc keeps M in registers)
+            for (int kc = 0; kc < NKC; ++kc) {
+                if (kc / (NKC / 2) != half) continue;    // (compile-time kc keeps M in registers)
                 uint4 hv, lv;
                 av_split(M[4 * kc + 0], hv.x, lv.x);
                 av_split(M[4 * kc + 1], hv.y, lv.y);
@@ -243,20 +275,21 @@ __global__ void __launch_bounds__(AV_THREADS, 1) k_adjoint_v(const __grid_consta
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            // epilogue: U^M_t = W_x sum_a M_a V[x, 16 t + a], two t per TMEM wait, two
-            // partial sums per t (columns past 16 P lie inside the group's 256 and are unused)
+            // epilogue: U^M_t = W_x sum_a M_a V[x, AC t + a], TT values of t per TMEM wait, two
+            // partial sums per t (columns past AC P lie inside the 512 and are unused)
             const float w = in ? __ldg(a.W + x) : 0.f;
             float* out = a.maps + (int64_t)(b0 + j) * a.P * a.npix + x;
-            for (int t0 = 8 * half; t0 < min(a.P, 8 * half + 8); t0 += 2) {
+            for (int t0 = t_begin; t0 < t_end; t0 += TT) {
                 uint32_t r[32];
-                av_ld32(lane_base + (uint32_t)(16 * t0), r);
+                if constexpr (AC == 12) av_ld24(lane_base + (uint32_t)(AC * t0), r);
+                else av_ld32(lane_base + (uint32_t)(AC * t0), r);
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
+                for (int i = 0; i < TT; ++i) {
                     float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-                    for (int q = 0; q < AV_PM / 2; ++q) {
-                        s0 = fmaf(M[q], __uint_as_float(r[16 * i + q]), s0);
-                        s1 = fmaf(M[q + 8], __uint_as_float(r[16 * i + q + 8]), s1);
+                    for (int q = 0; q < AC / 2; ++q) {
+                        s0 = fmaf(M[q], __uint_as_float(r[AC * i + q]), s0);
+                        s1 = fmaf(M[q + AC / 2], __uint_as_float(r[AC * i + q + AC / 2]), s1);
                     }
                     if (in && t0 + i < a.P) out[(int64_t)(t0 + i) * a.npix] = w * (s0 + s1);
                 }
@@ -280,12 +313,15 @@ cudaError_t launch_adjoint_v(Plan& pl, int B, const float* hk, float* maps, cuda
     if (B == 0) return cudaSuccess;
     // the map rows' pitch (npix floats) must be a multiple of 16 bytes for the tensor map
     if (!pl.adj_gops || B > pl.chunk || pl.P > AV_PM || pl.npix % 4 != 0) return cudaErrorInvalidValue;
-    k_adjv_gprep<<<B, 256, 0, st>>>(pl.P, pl.n_pair, hk, pl.adj_gops);
+    k_adjv_gprep<<<B, 256, 0, st>>>(pl.P, av_cols(pl.P), pl.n_pair, hk, pl.adj_gops);
     note_launch(pl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const size_t smem = 1024 + (size_t)AV_MAPS * AV_BMAP + (size_t)AV_GROUPS * AV_ABUF + (size_t)AV_STAGES * AV_MT;
-    e = cudaFuncSetAttribute(k_adjoint_v, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int AC = av_cols(pl.P), groups = AC == 16 ? AvShape<16>::GROUPS : AvShape<12>::GROUPS;
+    const size_t smem = 1024 + (size_t)AV_MAPS * AV_BMAP + (size_t)groups * AV_ABUF + (size_t)AV_STAGES * AV_MT;
+    auto kernel = AC == 8 ? k_adjoint_v<8> : (AC == 12 ? k_adjoint_v<12> : k_adjoint_v<16>);
+    const int threads = AC == 16 ? AvShape<16>::THREADS : AvShape<12>::THREADS;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     AdjVArgs a;
     a.P = pl.P;
@@ -312,7 +348,7 @@ cudaError_t launch_adjoint_v(Plan& pl, int B, const float* hk, float* maps, cuda
         const cuuint32_t box[2] = {128, (cuuint32_t)AV_PM};
         e = tma_map_f32(&mm, maps + (int64_t)a.b_first * pl.P * pl.npix, 2, dims, strides, box);
         if (e != cudaSuccess) return e;
-        k_adjoint_v<<<nq * a.G, AV_THREADS, smem, st>>>(mm, a);
+        kernel<<<nq * a.G, threads, smem, st>>>(mm, a);
         note_launch(pl);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
