@@ -452,7 +452,7 @@ cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cu
 // bytes) of its TL rows and TC columns at a time; the padding of 4 floats per row puts the
 // rows on different banks.  Synchronous staging through registers, one tile of 64 x 64 for
 // every size, took (us, linear term of one call) 290 at l_max = 32 with 6 modes and one map,
-// 2467 at l_max = 250 with 8 modes and 21 maps; now 28 and 183.
+// 2467 at l_max = 250 with 8 modes and 21 maps; now 23 and 141.
 __device__ __forceinline__ void lg_cp16(float* dst, const float* src, int bytes) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
@@ -582,32 +582,35 @@ static cudaError_t linear_gemm_launch(Plan& pl, const float* maps, int ncols, in
     return cudaGetLastError();
 }
 
-// The same sums where the outputs are few: 16 x 16 outputs per block, 2 x 2 per thread of two
-// compute warps, which do nothing but read and accumulate (a stage of LC_BK pixels is 4 LC_BK
-// FMAs deep per chain); two copy warps keep LC_ST stages in flight and multiply the panel's
-// pieces by W.  With copies, weights and sums in the same warps the chain advanced by one
-// pixel in 20 cycles.  Blocks alternate which warps compute, so that the compute warps of two
-// blocks on an SM sit on different sub-partitions.
-constexpr int LC_BK = 64, LC_ST = 4, LC_S = LC_BK + 4, LC_Q = LC_BK / 4;
-constexpr int LC_G = 4;                     // pieces per read-ahead group
-constexpr int LC_STAGE = 32 * LC_S;
-constexpr size_t LC_SMEM = (size_t)LC_ST * LC_STAGE * sizeof(float);
+// The same sums where the outputs are few: one compute warp per block, which does nothing but read
+// and accumulate, and one copy warp, which keeps LC_ST - 1 stages in flight and multiplies the
+// panel's pieces by W.  (With copies, weights and sums in the same warps a chain advanced by one
+// pixel in 20 clocks; here in 8.7 with one block per SM.)  A thread holds 2 rows x 2 columns: a
+// warp's 16-byte read occupies the shared-memory return path for four clocks whatever its lanes
+// share, so several blocks on an SM are bound by that path; blocks of 8 rows waste little of 21,
+// 36 or 55 pairs there (21 maps, l_max = 250, 8 modes: 183 us with 16 x 16 blocks, 141; 2 x 4
+// outputs per thread, with fewer bytes per output and fewer warps, 179).
+constexpr int LC_BK = 128, LC_ST = 4, LC_S = LC_BK + 4, LC_Q = LC_BK / 4, LC_R = 8;
+constexpr int LC_C = 16;                    // columns per block
+constexpr size_t LC_SMEM = (size_t)LC_ST * (LC_R + LC_C) * LC_S * sizeof(float);
 
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(64)
 k_linear_chain(int nrows, int ncols, int64_t npix, int64_t kchunk, const float* __restrict__ panel,
                const float* __restrict__ W, const float* __restrict__ maps, double* __restrict__ out) {
+    constexpr int LC_STAGE = (LC_R + LC_C) * LC_S;
+    constexpr int TC = LC_C / 8, G = 4;                      // columns per thread, pieces per read-ahead group
     extern __shared__ __align__(16) float lg_sm[];
-    const int r0 = blockIdx.x * 16, c0 = blockIdx.y * 16;
+    const int r0 = blockIdx.x * LC_R, c0 = blockIdx.y * LC_C;
     const int64_t k_begin = (int64_t)blockIdx.z * kchunk;
     const int64_t k_end = min(npix, k_begin + kchunk);
     const int nk = k_end > k_begin ? (int)((k_end - k_begin + LC_BK - 1) / LC_BK) : 0;
-    const int swap = (blockIdx.x + blockIdx.y + blockIdx.z) & 1;
-    const int role = (threadIdx.x / 64) ^ swap;              // 0: compute, 1: copy
-    const int tid = threadIdx.x % 64;
+    // blocks alternate which warp computes: two blocks' compute warps then sit on different sub-partitions
+    const bool copies = (threadIdx.x / 32 ^ (blockIdx.x + blockIdx.y + blockIdx.z)) & 1;
+    const int lane = threadIdx.x % 32;
     // barriers: 1 + s: stage s is filled; 1 + LC_ST + s: stage s has been read
-    if (role == 1) {
-        const int q = tid % LC_Q, lr = tid / LC_Q;           // pieces q of rows lr + RS u
-        constexpr int RS = 64 / LC_Q, NU = 16 / RS;
+    if (copies) {
+        constexpr int RS = 32 / LC_Q, NA = LC_R / RS, NB = LC_C / RS;
+        const int q = lane % LC_Q, lr = lane / LC_Q;         // pieces q of rows lr + RS u
         const float* pa = panel + (int64_t)(r0 + lr) * npix + k_begin + 4 * q;
         const float* pb = maps + (int64_t)(c0 + lr) * npix + k_begin + 4 * q;
         const float* pw = W + k_begin + 4 * q;
@@ -620,10 +623,14 @@ k_linear_chain(int nrows, int ncols, int64_t npix, int64_t kchunk, const float* 
                 const bool in = k_begin + off + 4 * q < k_end;
                 float* st = lg_sm + (k % LC_ST) * LC_STAGE + lr * LC_S + 4 * q;
 #pragma unroll
-                for (int u = 0; u < NU; ++u) {
-                    const bool oka = in && r0 + lr + RS * u < nrows, okb = in && c0 + lr + RS * u < ncols;
-                    lg_cp16(st + RS * u * LC_S, oka ? pa + off + u * step : panel, oka ? 16 : 0);
-                    lg_cp16(st + (16 + RS * u) * LC_S, okb ? pb + off + u * step : maps, okb ? 16 : 0);
+                for (int u = 0; u < NA; ++u) {
+                    const bool ok = in && r0 + lr + RS * u < nrows;
+                    lg_cp16(st + RS * u * LC_S, ok ? pa + off + u * step : panel, ok ? 16 : 0);
+                }
+#pragma unroll
+                for (int u = 0; u < NB; ++u) {
+                    const bool ok = in && c0 + lr + RS * u < ncols;
+                    lg_cp16(st + (LC_R + RS * u) * LC_S, ok ? pb + off + u * step : maps, ok ? 16 : 0);
                 }
                 if (in) wk = __ldg(reinterpret_cast<const float4*>(pw + off));
             }
@@ -639,71 +646,75 @@ k_linear_chain(int nrows, int ncols, int64_t npix, int64_t kchunk, const float* 
                 asm volatile("cp.async.wait_group %0;" ::"n"(LC_ST - 2) : "memory");
                 float* own = lg_sm + s * LC_STAGE + lr * LC_S + 4 * q;
 #pragma unroll
-                for (int u = 0; u < NU; ++u) {
+                for (int u = 0; u < NA; ++u) {
                     float4* v = reinterpret_cast<float4*>(own + RS * u * LC_S);
                     const float4 x = *v;
                     *v = make_float4(x.x * w[s].x, x.y * w[s].y, x.z * w[s].z, x.w * w[s].w);
                 }
                 __threadfence_block();
-                named_arrive(1 + s, 128);
+                named_arrive(1 + s, 64);
                 const int kn = k + LC_ST - 1;                // goes where step k - 1 was
-                if (k >= 1 && kn < nk) named_sync(1 + LC_ST + (s + LC_ST - 1) % LC_ST, 128);
+                if (k >= 1 && kn < nk) named_sync(1 + LC_ST + (s + LC_ST - 1) % LC_ST, 64);
                 issue(kn, w[(s + LC_ST - 1) % LC_ST]);
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         return;
     }
-    const int rg = tid % 4 + 4 * ((tid / 16) % 2), cg = (tid / 4) % 4 + 4 * (tid / 32);   // rows rg, rg + 8; columns cg, cg + 8
-    float acc[2][2] = {};
+    const int rg = lane % 4, cg = lane / 4;                  // rows rg, rg + 4; columns cg + 8 i
+    float acc[2][TC];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < TC; ++j) acc[i][j] = 0.f;
     for (int k = 0; k < nk; ++k) {
         const int s = k % LC_ST;
-        named_sync(1 + s, 128);
+        named_sync(1 + s, 64);
         const float* sa = lg_sm + s * LC_STAGE + rg * LC_S;
-        const float* sb = lg_sm + s * LC_STAGE + (16 + cg) * LC_S;
-        // groups of LC_G pieces: the next group's reads are issued before this group's sums
-        float4 a[2][LC_G][2], b[2][LC_G][2];
+        const float* sb = lg_sm + s * LC_STAGE + (LC_R + cg) * LC_S;
+        // the next group's reads are issued before this group's sums
+        float4 a[2][G][2], b[2][G][TC];
         auto read = [&](int h, int g) {
 #pragma unroll
-            for (int p = 0; p < LC_G; ++p)
+            for (int p = 0; p < G; ++p) {
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    a[h][p][i] = *reinterpret_cast<const float4*>(sa + 8 * i * LC_S + 4 * (g * LC_G + p));
-                    b[h][p][i] = *reinterpret_cast<const float4*>(sb + 8 * i * LC_S + 4 * (g * LC_G + p));
-                }
+                for (int i = 0; i < 2; ++i) a[h][p][i] = *reinterpret_cast<const float4*>(sa + 4 * i * LC_S + 4 * (g * G + p));
+#pragma unroll
+                for (int i = 0; i < TC; ++i) b[h][p][i] = *reinterpret_cast<const float4*>(sb + 8 * i * LC_S + 4 * (g * G + p));
+            }
         };
         read(0, 0);
 #pragma unroll
-        for (int g = 0; g < LC_Q / LC_G; ++g) {
+        for (int g = 0; g < LC_Q / G; ++g) {
             const int h = g & 1;
-            if (g + 1 < LC_Q / LC_G) read(h ^ 1, g + 1);
+            if (g + 1 < LC_Q / G) read(h ^ 1, g + 1);
 #pragma unroll
-            for (int p = 0; p < LC_G; ++p) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[h][p][i].x, b[h][p][j].x, acc[i][j]);
+            for (int p = 0; p < G; ++p) {
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[h][p][i].y, b[h][p][j].y, acc[i][j]);
+                    for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(a[h][p][i].x, b[h][p][j].x, acc[i][j]);
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[h][p][i].z, b[h][p][j].z, acc[i][j]);
+                    for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(a[h][p][i].y, b[h][p][j].y, acc[i][j]);
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[h][p][i].w, b[h][p][j].w, acc[i][j]);
+                    for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(a[h][p][i].z, b[h][p][j].z, acc[i][j]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(a[h][p][i].w, b[h][p][j].w, acc[i][j]);
             }
         }
-        if (k + LC_ST < nk) named_arrive(1 + LC_ST + s, 128);    // the copy of step k + LC_ST waits for this
+        if (k + LC_ST < nk) named_arrive(1 + LC_ST + s, 64);     // the copy of step k + LC_ST waits for this
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int r = r0 + rg + 8 * i, c = c0 + cg + 8 * j;
+        for (int j = 0; j < TC; ++j) {
+            const int r = r0 + rg + 4 * i, c = c0 + cg + 8 * j;
             if (r < nrows && c < ncols) out[((int64_t)blockIdx.z * nrows + r) * ncols + c] = (double)acc[i][j];
         }
 }
@@ -716,15 +727,15 @@ cudaError_t launch_linear_gemm(Plan& pl, const float* maps, int B, double* parti
         return (int64_t)((pl.n_pair + bm - 1) / bm) * ((ncols + bn - 1) / bn) * pl.lin_ksplit;
     };
     // The largest tile that still fills the SMs: a block of the larger tiles is two warps, and an
-    // SM needs about eight of them before its FP32 units are busy (136 pairs x 16 maps on 501 x
-    // 1024 pixels with one block per SM, us: 64 x 64 1507, 32 x 32 892); below two blocks of 32 x
-    // 32 per SM the chains' own latency is the bound (55 pairs, 8 maps of 10 modes: 452 with
-    // 32 x 32 tiles, 370 with k_linear_chain).
+    // SM needs about eight of them before its FP32 units are busy (136 pairs x 16 modes x 8 maps on
+    // 501 x 1024 pixels, us: 64 x 64 1507, 32 x 32 889, chains 1004); with fewer blocks of 32 x 32
+    // the chains' own latency is the bound (55 pairs, 8 maps of 10 modes, 1.2 blocks per SM: 452
+    // with 32 x 32 tiles, 309 with k_linear_chain).
     if (blocks(64, 64) >= 4 * (int64_t)pl.nsm) return linear_gemm_launch<64, 64, 8, 8, 16, 4>(pl, maps, ncols, kchunk, partial, st);
-    if (blocks(32, 32) >= 2 * (int64_t)pl.nsm) return linear_gemm_launch<32, 32, 4, 4, 32, 4>(pl, maps, ncols, kchunk, partial, st);
+    if (blocks(32, 32) >= 3 * (int64_t)pl.nsm) return linear_gemm_launch<32, 32, 4, 4, 32, 4>(pl, maps, ncols, kchunk, partial, st);
     const cudaError_t e = cudaFuncSetAttribute(k_linear_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LC_SMEM);
     if (e != cudaSuccess) return e;
-    k_linear_chain<<<dim3((pl.n_pair + 15) / 16, (ncols + 15) / 16, pl.lin_ksplit), 128, LC_SMEM, st>>>(
+    k_linear_chain<<<dim3((pl.n_pair + LC_R - 1) / LC_R, (ncols + LC_C - 1) / LC_C, pl.lin_ksplit), 64, LC_SMEM, st>>>(
         pl.n_pair, ncols, pl.npix, kchunk, pl.pair_mean, pl.W, maps, partial);
     note_launch(pl);
     return cudaGetLastError();
