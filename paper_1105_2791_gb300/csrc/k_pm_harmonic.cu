@@ -334,32 +334,57 @@ __global__ void __launch_bounds__(LH_THREADS) k_linh_s(int L, int n_pair, int B,
 // FP64 sum: each product's rounding error is recovered exactly by an FMA and each
 // addition's by Knuth's two-sum, the errors are added up beside the sum, and every block
 // goes to an FP64 accumulator.  (FP64 throughput on sm_103a is near 1 TF/s; a plain FP64
-// chain per output took 0.84 ms at l_max = 2000, 32 maps.)
-__global__ void k_linh_g(int L, int P, int n_pair, int B, const float* __restrict__ filt, const float* __restrict__ S,
-                         double* __restrict__ lin) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B * n_pair * P) return;
-    const int t = i % P, bc = i / P, c = bc % n_pair, b = bc / n_pair;
-    const float* srow = S + ((int64_t)b * n_pair + c) * (L + 1);
-    const float* frow = filt + (int64_t)t * (L + 1);
-    double acc = 0.0;
-    for (int l0 = 0; l0 <= L; l0 += 32) {
-        float sum = 0.f, err = 0.f;
-        const int l1 = min(L + 1, l0 + 32);
-        for (int l = l0; l < l1; ++l) {
-            const float f = frow[l], v = srow[l];
-            // _rn intrinsics: no operation below may be contracted into an FMA
-            const float p = __fmul_rn(f, v);
-            const float pe = fmaf(f, v, -p);        // f v - p exactly
-            const float s2 = __fadd_rn(sum, p);     // two-sum: sum + p = s2 + se exactly
-            const float z = __fsub_rn(s2, sum);
-            const float se = __fadd_rn(__fsub_rn(sum, __fsub_rn(s2, z)), __fsub_rn(p, z));
-            sum = s2;
-            err = __fadd_rn(err, __fadd_rn(se, pe));
+// chain per output took 0.84 ms at l_max = 2000, 32 maps.)  A block takes all t of up to
+// LG2_OUT / P pairs of one map; each 32 values of l of its rows of S and of f come through shared memory while
+// the 32 before are summed (read by each thread as it went, the chain waited for every load: 64
+// maps, l_max = 500, 10 modes 54 us, now 30; 12 maps, l_max = 1000, 16 modes 120, now 39).
+constexpr int LG2_OUT = 256;
+
+__global__ void __launch_bounds__(LG2_OUT) k_linh_g(int L, int P, int n_pair, int B, int cpb, const float* __restrict__ filt,
+                                                    const float* __restrict__ S, double* __restrict__ lin) {
+    extern __shared__ float lg2_sm[];                       // [2][P + cpb][33]: rows of f, then of S
+    const int b = blockIdx.x, c0 = blockIdx.y * cpb;
+    const int tid = threadIdx.x, t = tid % P, cl = tid / P;
+    const bool active = cl < cpb && c0 + cl < n_pair;
+    const int nc = min(cpb, n_pair - c0);
+    const float* Sb = S + ((int64_t)b * n_pair + c0) * (L + 1);
+    auto stage = [&](int h, int l0) {                       // rows of f, then of S, 32 values each; zero past L
+        for (int i = tid; i < (P + nc) * 32; i += LG2_OUT) {
+            const int r = i / 32, k = i % 32, l = l0 + k;
+            float* dst = lg2_sm + (h * (P + cpb) + r) * 33 + k;
+            const float* src = (r < P ? filt + (int64_t)r * (L + 1) : Sb + (int64_t)(r - P) * (L + 1)) + l;
+            const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(l <= L ? src : filt), "r"(l <= L ? 4 : 0)
+                         : "memory");
         }
-        acc += (double)sum + (double)err;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    double acc = 0.0;
+    stage(0, 0);
+    int h = 0;
+    for (int l0 = 0; l0 <= L; l0 += 32, h ^= 1) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        if (l0 + 32 <= L) stage(h ^ 1, l0 + 32);
+        if (active) {
+            const float* row = lg2_sm + h * (P + cpb) * 33;
+            float sum = 0.f, err = 0.f;
+            const int n = min(32, L + 1 - l0);
+            for (int k = 0; k < n; ++k) {
+                const float f = row[t * 33 + k], v = row[(P + cl) * 33 + k];
+                // _rn intrinsics: no operation below may be contracted into an FMA
+                const float p = __fmul_rn(f, v);
+                const float pe = fmaf(f, v, -p);        // f v - p exactly
+                const float s2 = __fadd_rn(sum, p);     // two-sum: sum + p = s2 + se exactly
+                const float z = __fsub_rn(s2, sum);
+                const float se = __fadd_rn(__fsub_rn(sum, __fsub_rn(s2, z)), __fsub_rn(p, z));
+                sum = s2;
+                err = __fadd_rn(err, __fadd_rn(se, pe));
+            }
+            acc += (double)sum + (double)err;
+        }
     }
-    lin[(int64_t)c * (B * P) + b * P + t] = acc;
+    if (active) lin[(int64_t)(c0 + cl) * (B * P) + b * P + t] = acc;
 }
 
 cudaError_t launch_linear_harmonic(Plan& pl, const float2* alm, int B, double* lin, cudaStream_t st) {
@@ -370,8 +395,9 @@ cudaError_t launch_linear_harmonic(Plan& pl, const float2* alm, int B, double* l
     note_launch(pl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int n = B * pl.n_pair * pl.P;
-    k_linh_g<<<(n + 127) / 128, 128, 0, st>>>(pl.lmax, pl.P, pl.n_pair, B, pl.filt, pl.adj_pmk, lin);
+    const int cpb = std::min(LG2_OUT / pl.P, pl.n_pair);    // at most 36 pairs (7 modes): 11 KB of shared memory
+    k_linh_g<<<dim3(B, (pl.n_pair + cpb - 1) / cpb), LG2_OUT, 2 * (size_t)(pl.P + cpb) * 33 * sizeof(float), st>>>(
+        pl.lmax, pl.P, pl.n_pair, B, cpb, pl.filt, pl.adj_pmk, lin);
     note_launch(pl);
     return cudaGetLastError();
 }
