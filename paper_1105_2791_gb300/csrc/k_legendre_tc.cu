@@ -104,6 +104,16 @@ struct PrepArgs {
     char* out;                     // [n_groups][total_bkb][2][N][128 bytes]
 };
 
+// Spans in flight per pair of orders: 5, 9, 17 and 33 measured alike; 9 leaves a CTA four at l_max = 2000.
+constexpr int PREPB_X = 9;
+
+// Bound by the bytes it writes: 4 per value of B, hi and lo.  A CTA takes spans of 2 KPS
+// consecutive l of one map group, both parities at once, so that its a_lm reads are whole lines;
+// a thread makes the re and im columns of one (map, mode) from one read of each value.  Orders m
+// and L - m share a row of the grid: together they have nearly the same number of spans whatever
+// m, and no CTA starts without work.  64 maps, l_max = 500, 10 modes: 158 us (643 MB written, 0.6
+// of measured HBM); with one parity per CTA, one column per thread and the scales fetched before
+// the a_lm 191.  12 maps, l_max = 1000, 16 modes: 195 -> 185; l_max = 2000, 8 maps: 367 both (2 GB, 0.82).
 template <int PREC>
 __global__ void __launch_bounds__(256) k_tc_prep_b(PrepArgs a) {
     using S = Split<PREC>;
@@ -111,64 +121,66 @@ __global__ void __launch_bounds__(256) k_tc_prep_b(PrepArgs a) {
     constexpr int KPS = TC_KB / S::E;
     constexpr int CM = 16 / S::E;
     constexpr int NKC = TC_KB / 16;
-    __shared__ float2 s_a[TC_MAX_MAPS * 32];
-    __shared__ float s_f[64 * 16];
-    __shared__ float s_scale[TC_MAX_MAPS];
-    __shared__ int s_dec[16 * 16];                              // per column n: (map row of s_a, p, Re/Im)
-    const int N = 2 * a.P * a.G;
-    const int b_tile = N * TC_KB;
-    const int m = blockIdx.y >> 1, pi = blockIdx.y & 1, g = blockIdx.z;
-    const int nkb = tc_nkb(a.L, m, pi, KPS);
-    const int64_t base_m = d_alm_index(m, m, a.L);
-    if (threadIdx.x < a.G) {
-        const int b = g * a.G + threadIdx.x;
-        s_scale[threadIdx.x] = (b < a.B) ? exp2f((float)tc_scale_exp(a.amax[b])) : 0.f;
-    }
-    // column n = (map bl, p, Re/Im) = 2 (bl P + p) + comp, decoded once per CTA
-    for (int n = threadIdx.x; n < N; n += blockDim.x)
-        s_dec[n] = ((n / (2 * a.P)) * KPS) << 16 | ((n / 2) % a.P) << 1 | (n & 1);
-    // this thread's first (chunk column, n) and its stride over c = kc N + n, divided once
-    const int kc0 = threadIdx.x / N, n0 = threadIdx.x % N;
-    const int dkc = blockDim.x / N, dn = blockDim.x % N;
-    for (int kb = blockIdx.x; kb < nkb; kb += gridDim.x) {
-        const int l0 = m + pi + 2 * kb * KPS;                   // l of K index k: l0 + 2 k
+    constexpr int SPAN = 2 * KPS;                               // l per span: KPS of each parity
+    __shared__ float2 s_a[TC_MAX_MAPS * (SPAN + 1)];
+    __shared__ float s_f[SPAN * 17];
+    __shared__ int s_dec[8 * 16];                               // per column pair: row of s_a, p
+    const int NP = a.P * a.G;                                   // column pairs (map bl, p) of (re, im)
+    const int b_tile = 2 * NP * TC_KB;
+    const int g = blockIdx.z;
+    const int m_lo = blockIdx.y, m_hi = a.L - blockIdx.y;       // equal for the middle order of an even L
+    const int n_lo = tc_nkb(a.L, m_lo, 0, KPS), n_hi = m_hi > m_lo ? tc_nkb(a.L, m_hi, 0, KPS) : 0;
+    for (int n = threadIdx.x; n < NP; n += blockDim.x) s_dec[n] = (n / a.P * (SPAN + 1)) << 8 | n % a.P;
+    // this thread's first (parity and chunk column q, pair n) and its stride over c = q NP + n, divided once
+    const int q0 = threadIdx.x / NP, n0 = threadIdx.x % NP;
+    const int dq = blockDim.x / NP, dn = blockDim.x % NP;
+    for (int s = blockIdx.x; s < n_lo + n_hi; s += gridDim.x) {
+        const int m = s < n_lo ? m_lo : m_hi, kb = s < n_lo ? s : s - n_lo;
+        const int l0 = m + kb * SPAN, nl = min(SPAN, a.L + 1 - l0);
         __syncthreads();
-        for (int i = threadIdx.x; i < a.G * KPS; i += blockDim.x) {
-            const int bl = i / KPS, k = i % KPS;
-            const int b = g * a.G + bl, l = l0 + 2 * k;
+        const float2* arow = a.alm + d_alm_index(m, m, a.L) + (l0 - m);
+#pragma unroll 4
+        for (int i = threadIdx.x; i < a.G * SPAN; i += blockDim.x) {
+            const int bl = i / SPAN, k = i % SPAN, b = g * a.G + bl;
             float2 v = make_float2(0.f, 0.f);
-            if (b < a.B && l <= a.L) {
-                v = a.alm[(int64_t)b * a.n_alm + base_m + (l - m)];
-                v.x *= s_scale[bl];
-                v.y *= s_scale[bl];
+            if (b < a.B && k < nl) {
+                const float scale = exp2f((float)tc_scale_exp(a.amax[b]));
+                v = arow[(int64_t)b * a.n_alm + k];
+                v.x *= scale;
+                v.y *= scale;
             }
-            s_a[i] = v;
+            s_a[bl * (SPAN + 1) + k] = v;
         }
-        for (int i = threadIdx.x; i < KPS * 16; i += blockDim.x) {
-            const int k = i / 16, p = i % 16, l = l0 + 2 * k;
-            s_f[i] = (p < a.P && l <= a.L) ? a.filt[(int64_t)p * (a.L + 1) + l] : 0.f;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < a.P * SPAN; i += blockDim.x) {
+            const int p = i / SPAN, k = i % SPAN;
+            s_f[k * 17 + p] = k < nl ? a.filt[(int64_t)p * (a.L + 1) + l0 + k] : 0.f;
         }
         __syncthreads();
-        char* bt = a.out + ((int64_t)g * a.total_bkb + a.bblk_base[2 * m + pi] + kb) * (int64_t)(2 * b_tile);
-        for (int kc = kc0, n = n0; kc < NKC;) {
-            const int dec = s_dec[n];
-            const int arow = dec >> 16, p = (dec >> 1) & 0x7fff, comp = dec & 1;
-            T hv[CM], lv[CM];
+        char* bt = a.out + ((int64_t)g * a.total_bkb + kb) * (int64_t)(2 * b_tile);
+        const int64_t at0 = a.bblk_base[2 * m] * (2 * b_tile), at1 = a.bblk_base[2 * m + 1] * (2 * b_tile);
+        const int nq = kb < tc_nkb(a.L, m, 1, KPS) ? 2 * NKC : NKC;
+        for (int q = q0, n = n0; q < nq;) {
+            const int pi = q / NKC, kc = q % NKC;
+            const int dec = s_dec[n], p = dec & 255;
+            const float2* av = s_a + (dec >> 8) + 2 * kc * CM + pi;
+            const float* fv = s_f + (2 * kc * CM + pi) * 17 + p;
+            T hr[CM], hm[CM], lr[CM], lm[CM];
 #pragma unroll
             for (int i = 0; i < CM; ++i) {
-                const int k = kc * CM + i;
-                const float2 av = s_a[arow + k];
-                const float x = s_f[k * 16 + p] * (comp ? av.y : av.x);
-                S::split(x, hv[i], lv[i]);
+                const float2 v = av[2 * i];
+                const float f = fv[2 * i * 17];
+                S::split(f * v.x, hr[i], lr[i]);
+                S::split(f * v.y, hm[i], lm[i]);
             }
-            const int off = (n >> 3) * TC_SBO + kc * 128 + (n & 7) * 16;
-            *reinterpret_cast<uint4*>(bt + off) = *reinterpret_cast<const uint4*>(hv);
-            *reinterpret_cast<uint4*>(bt + b_tile + off) = *reinterpret_cast<const uint4*>(lv);
-            kc += dkc;
+            char* dst = bt + (pi ? at1 : at0) + (n >> 2) * TC_SBO + kc * 128 + (n & 3) * 32;
+            st_pair(dst, hr, hm);
+            st_pair(dst + b_tile, lr, lm);
+            q += dq;
             n += dn;
-            if (n >= N) {
-                n -= N;
-                ++kc;
+            if (n >= NP) {
+                n -= NP;
+                ++q;
             }
         }
     }
@@ -525,8 +537,8 @@ void free_tc_tables(Plan& pl) {
 template <int PREC>
 static cudaError_t launch_tc(const Plan& pl, const PrepArgs& pa, const TcArgs& args, int part, cudaStream_t st) {
     if (part & 1) {
-        const int maxkb = tc_nkb(pl.lmax, 0, 0, kps_for(pl.prec));
-        dim3 grid(std::min(maxkb, 8), 2 * (pl.lmax + 1), pa.n_groups);
+        const int spans = tc_nkb(pl.lmax, 0, 0, kps_for(pl.prec)) + 1;      // of orders m and L - m
+        dim3 grid(std::min(spans, PREPB_X), pl.lmax / 2 + 1, pa.n_groups);
         k_tc_prep_b<PREC><<<grid, 256, 0, st>>>(pa);
         note_launch(pl);
         cudaError_t e = cudaGetLastError();

@@ -153,10 +153,8 @@ __global__ void __launch_bounds__(256) k_tc_prep_adj(AdjPrepArgs a) {
             }
             const int n = 2 * q;                             // Re row; the Im row n + 1 is 16 bytes on
             const int off = (n / 8) * TC_SBO + kc * 128 + (n % 8) * 16;
-            *reinterpret_cast<uint4*>(bt + off) = *reinterpret_cast<const uint4*>(hr);
-            *reinterpret_cast<uint4*>(bt + off + 16) = *reinterpret_cast<const uint4*>(hm);
-            *reinterpret_cast<uint4*>(bt + b_tile + off) = *reinterpret_cast<const uint4*>(lr);
-            *reinterpret_cast<uint4*>(bt + b_tile + off + 16) = *reinterpret_cast<const uint4*>(lm);
+            st_pair(bt + off, hr, hm);
+            st_pair(bt + b_tile + off, lr, lm);
         }
     }
 }

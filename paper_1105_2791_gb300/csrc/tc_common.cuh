@@ -172,6 +172,16 @@ __device__ __forceinline__ int tc_scale_exp(unsigned amax_bits) {
     return max(-120, min(120, 141 - e));
 }
 
+// 32 bytes in one store (p 32-byte aligned): the 16 of two neighbouring operand rows, a whole sector.
+__device__ __forceinline__ void st_pair(char* p, const void* row0, const void* row1) {
+    uint32_t v[8];
+    memcpy(v, row0, 16);
+    memcpy(v + 4, row1, 16);
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
+                 "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
 template <int E>
 struct ElemT;
 template <>
