@@ -90,12 +90,12 @@ __global__ void __launch_bounds__(256) k_alm_amax(int L, const float* __restrict
 }
 
 // ------------------------------------------------------------------ B operand blocks
-// Stage block (g, m, pi, kb) of the filtered a_lm for maps G g .. G g + G - 1 (G maps per
-// group, the plan's tunable): [hi tile, lo tile], each N = 2 P G rows (b, p, re/im) x TC_KB
+// Stage block (g, m, pi, kb) of the filtered a_lm for maps G g .. G g + G - 1 (at most the plan's
+// tunable per group): [hi tile, lo tile], each N >= 2 P G rows (b, p, re/im; padded to 16) x TC_KB
 // bytes of K (KPS values l = m + pi + 2 (kb KPS + k)), the same core-matrix layout the MMA
 // reads.  Built once per chunk and shared by every ring tile.
 struct PrepArgs {
-    int L, P, B, G, n_groups;
+    int L, P, B, G, N, n_groups;
     int64_t n_alm, total_bkb;      // stage blocks per map group
     const int64_t* bblk_base;      // [2 (L+1)] first stage block of (m, parity)
     const float* filt;             // [P][L+1]
@@ -125,12 +125,14 @@ __global__ void __launch_bounds__(256) k_tc_prep_b(PrepArgs a) {
     __shared__ float2 s_a[TC_MAX_MAPS * (SPAN + 1)];
     __shared__ float s_f[SPAN * 17];
     __shared__ int s_dec[8 * 16];                               // per column pair: row of s_a, p
-    const int NP = a.P * a.G;                                   // column pairs (map bl, p) of (re, im)
-    const int b_tile = 2 * NP * TC_KB;
+    const int NP = a.N / 2;                                     // column pairs (map bl, p) of (re, im), padded to 8
+    const int b_tile = a.N * TC_KB;
     const int g = blockIdx.z;
     const int m_lo = blockIdx.y, m_hi = a.L - blockIdx.y;       // equal for the middle order of an even L
     const int n_lo = tc_nkb(a.L, m_lo, 0, KPS), n_hi = m_hi > m_lo ? tc_nkb(a.L, m_hi, 0, KPS) : 0;
-    for (int n = threadIdx.x; n < NP; n += blockDim.x) s_dec[n] = (n / a.P * (SPAN + 1)) << 8 | n % a.P;
+    for (int n = threadIdx.x; n < NP; n += blockDim.x)
+        s_dec[n] = n < a.P * a.G ? (n / a.P * (SPAN + 1)) << 8 | n % a.P : 16;
+    for (int k = threadIdx.x; k < SPAN; k += blockDim.x) s_f[k * 17 + 16] = 0.f;   // the padded pairs' filter
     // this thread's first (parity and chunk column q, pair n) and its stride over c = q NP + n, divided once
     const int q0 = threadIdx.x / NP, n0 = threadIdx.x % NP;
     const int dq = blockDim.x / NP, dn = blockDim.x % NP;
@@ -211,7 +213,7 @@ __device__ __forceinline__ void tmem_ld16x4(uint32_t a0, uint32_t a1, uint32_t a
 #undef TC_LD16
 
 struct TcArgs {
-    int L, P, R, R_half, RH, n_rt, B, G, n_groups;
+    int L, P, R, R_half, RH, n_rt, B, G, N, n_groups;
     int64_t n_items, total_bkb;
     const char* table;             // pre-tiled A blocks
     const int64_t* blk_base;       // [2 (L+1)] first A block of (m, parity)
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_legendre_tc(TcArgs a) {
     constexpr bool TF32 = (PREC == MODAL_3XTF32);
     constexpr int KPS = TC_KB / S::E;     // K values per stage
     constexpr int NKC = TC_KB / 16;       // core matrices along K per stage
-    const int N = 2 * a.P * a.G;          // 2 (re, im) x P x G maps
+    const int N = a.N;                    // 2 (re, im) x P x G maps, padded to 16
     const int b_tile = N * TC_KB;         // bytes of one B tile
     const uint32_t stage_tx = TC_A_STAGE + 2 * b_tile;
 
@@ -373,7 +375,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_legendre_tc(TcArgs a) {
             tc_fence_after();
             const int jn = rt * 128 + quarter * 32 + lane;   // TMEM lane = ring pair within the tile
             const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
-            const int cp_valid = (a.B - g * a.G) * a.P;       // column pairs that belong to real maps
+            const int cp_valid = min(a.G, a.B - g * a.G) * a.P;   // column pairs of this group's maps
             float2* base = a.delta + ((int64_t)g * a.G * a.P) * row_stride + (int64_t)(2 * m + pi) * a.RH + jn;
             auto store_block = [&](int blk, const float* d) {
                 const int cp0 = blk * 8;
@@ -571,8 +573,9 @@ cudaError_t launch_legendre_tc(const Plan& pl, const float2* alm, int B, float2*
     pa.L = pl.lmax;
     pa.P = pl.P;
     pa.B = B;
-    pa.G = pl.tc_maps;
-    pa.n_groups = (B + pa.G - 1) / pa.G;
+    pa.n_groups = (B + pl.tc_maps - 1) / pl.tc_maps;
+    pa.G = (B + pa.n_groups - 1) / pa.n_groups;             // groups of equal size: BALANCE
+    pa.N = tc_cols(pa.P, pa.G);
     pa.n_alm = pl.n_alm;
     pa.total_bkb = pl.tc.total_bkb;
     pa.bblk_base = pl.tc.d_bkb_off;
@@ -589,6 +592,7 @@ cudaError_t launch_legendre_tc(const Plan& pl, const float2* alm, int B, float2*
     a.n_rt = pl.tc.n_rt;
     a.B = B;
     a.G = pa.G;
+    a.N = pa.N;
     a.n_groups = pa.n_groups;
     a.n_items = (int64_t)(pl.lmax + 1) * 2 * a.n_rt * a.n_groups;
     a.total_bkb = pl.tc.total_bkb;

@@ -84,7 +84,7 @@ __global__ void k_ut_amax(int L, int P, int R_half, int RH, const float2* __rest
 }
 
 struct AdjPrepArgs {
-    int L, P, R_half, RH, B, nkb;
+    int L, P, R_half, RH, B, G, nkb;
     const float2* ut;              // [B][P][L+1][2][RH]
     const unsigned* amax;
     char* out;                     // [(g (L+1) + m) 2 + pi][kb][2][N][128 bytes]
@@ -103,14 +103,15 @@ __global__ void __launch_bounds__(256) k_tc_prep_adj(AdjPrepArgs a) {
     constexpr int CM = 16 / S::E;
     constexpr int NKC = TC_KB / 16;
     static_assert(CM % 2 == 0, "CM values of U~ are read as float4 pairs");
-    __shared__ float s_scale[TC_MAPS];
-    const int N = 16 * a.P;
+    __shared__ float s_scale[TC_MAPS + 8];                 // 0 for the rows that pad N (at most 7, P = 1)
+    const int N = tc_cols(a.P, a.G);
     const int NQ = N / 2;                                  // (bl, t) rows
     const int b_tile = N * TC_KB;
     const int m = blockIdx.y >> 1, pi = blockIdx.y & 1, g = blockIdx.z;
-    if (threadIdx.x < TC_MAPS) {
-        const int b = g * TC_MAPS + threadIdx.x;
-        s_scale[threadIdx.x] = (b < a.B) ? exp2f((float)tc_scale_exp(a.amax[b])) : 0.f;
+    const int b_end = min(a.B, (g + 1) * a.G);
+    if (threadIdx.x < TC_MAPS + 8) {
+        const int b = g * a.G + threadIdx.x;
+        s_scale[threadIdx.x] = (b < b_end) ? exp2f((float)tc_scale_exp(a.amax[b])) : 0.f;
     }
     __syncthreads();
     for (int kb = blockIdx.x; kb < a.nkb; kb += gridDim.x) {
@@ -118,11 +119,11 @@ __global__ void __launch_bounds__(256) k_tc_prep_adj(AdjPrepArgs a) {
         for (int c = threadIdx.x; c < NKC * NQ; c += blockDim.x) {
             const int kc = c % NKC, q = c / NKC;           // the NKC threads of a row read it contiguously
             const int bl = q / a.P, t = q % a.P;
-            const int b = g * TC_MAPS + bl;
+            const int b = g * a.G + bl;
             const float sc = s_scale[bl];
             const int j0 = kb * KPS + kc * CM;
             float re[CM], im[CM];
-            if (b < a.B && j0 + CM <= a.R_half) {
+            if (b < b_end && j0 + CM <= a.R_half) {
                 // whole core-matrix row inside the ring range: 16-byte loads (RH is a multiple of 32)
                 const float4* u4 = reinterpret_cast<const float4*>(
                     a.ut + ((((int64_t)(b * a.P + t)) * (a.L + 1) + m) * 2 + pi) * a.RH + j0);
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(256) k_tc_prep_adj(AdjPrepArgs a) {
                 for (int i = 0; i < CM; ++i) {
                     const int j = j0 + i;
                     float2 v = make_float2(0.f, 0.f);
-                    if (b < a.B && j < a.R_half) v = u[j];
+                    if (b < b_end && j < a.R_half) v = u[j];
                     re[i] = v.x * sc;
                     im[i] = v.y * sc;
                 }
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(256) k_tc_prep_adj(AdjPrepArgs a) {
 
 // ------------------------------------------------------------------ main kernel
 struct AdjArgs {
-    int L, P, B, n_groups, nkb;
+    int L, P, B, G, n_groups, nkb;
     int64_t n_items, n_alm;
     const int64_t* item_base;      // [2 (L+1) + 1] prefix sums of l tiles over (m, pi)
     const char* table;             // transposed lambda blocks
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(TA_THREADS, 1) k_legendre_tc_adj(AdjArgs a) {
     using S = Split<PREC>;
     constexpr bool TF32 = (PREC == MODAL_3XTF32);
     constexpr int NKC = TC_KB / 16;
-    const int N = 16 * a.P;
+    const int N = tc_cols(a.P, a.G);
     const int b_tile = N * TC_KB;
     const uint32_t stage_tx = TC_A_STAGE + 2 * b_tile;
 
@@ -304,8 +305,8 @@ __global__ void __launch_bounds__(TA_THREADS, 1) k_legendre_tc_adj(AdjArgs a) {
             ta_item(a, item, m, pi, lt, g);
             const int l = m + pi + 2 * (lt * 128 + quarter * 32 + lane);
             float inv_lane = 0.f;
-            if (lane < TC_MAPS && g * TC_MAPS + lane < a.B)
-                inv_lane = exp2f((float)-tc_scale_exp(a.amax[g * TC_MAPS + lane])) * lam_inv;
+            if (lane < a.G && g * a.G + lane < a.B)
+                inv_lane = exp2f((float)-tc_scale_exp(a.amax[g * a.G + lane])) * lam_inv;
             float* my_f = sF + (threadIdx.x - 64) * 17;      // this lane's f_t(l), t < P
             for (int t = 0; t < a.P; ++t) my_f[t] = (l <= a.L) ? a.filt[(int64_t)t * (a.L + 1) + l] : 0.f;
             bool ok = !*abort_flag && mbar_wait(tmem_full, nitem & 1, abort_flag, a.err);
@@ -318,7 +319,7 @@ __global__ void __launch_bounds__(TA_THREADS, 1) k_legendre_tc_adj(AdjArgs a) {
             const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
             float acc_re = 0.f, acc_im = 0.f;
             int bl = 0, t = 0;
-            for (int blk = 0; blk < a.P; ++blk) {                // N = 16 P columns in blocks of 16
+            for (int blk = 0; blk < N / 16; ++blk) {             // N columns in blocks of 16
                 float d[16], d2[16];
                 tmem_ld16(lane_addr + blk * 16, d);
                 if (S::PRODUCTS == 3) {
@@ -334,8 +335,8 @@ __global__ void __launch_bounds__(TA_THREADS, 1) k_legendre_tc_adj(AdjArgs a) {
                     if (++t == a.P) {
                         // map bl complete
                         const float inv = __shfl_sync(0xffffffffu, inv_lane, bl);
-                        const int b = g * TC_MAPS + bl;
-                        if (l <= a.L && b < a.B) {
+                        const int b = g * a.G + bl;
+                        if (l <= a.L && bl < a.G && b < a.B) {
                             const float cm = (m == 0) ? 1.f : 2.f;
                             a.grad[(int64_t)b * a.n_alm + d_alm_index(l, m, a.L)] =
                                 make_float2(cm * acc_re * inv, (m == 0) ? 0.f : cm * acc_im * inv);
@@ -488,6 +489,7 @@ cudaError_t launch_legendre_adjoint_tc(const Plan& pl, const float2* ut, int B, 
     a.P = pl.P;
     a.B = B;
     a.n_groups = (B + TC_MAPS - 1) / TC_MAPS;
+    a.G = pa.G = (B + a.n_groups - 1) / a.n_groups;         // groups of equal size, as in the forward sums
     a.nkb = pl.tca.nkb;
     a.n_items = pl.tca.n_lt_total * a.n_groups;
     a.n_alm = pl.n_alm;

@@ -10,7 +10,7 @@
 
 namespace modal {
 
-constexpr int TC_MAPS = 8;                 // maps per work item of the adjoint Legendre kernel (N = 16 P)
+constexpr int TC_MAPS = 8;                 // most maps per work item of the adjoint Legendre kernel (N <= 16 P)
 constexpr int TC_MAX_MAPS = 32;            // most maps per work item of the forward kernel (tunable, N = 2 P G <= 256)
 constexpr int TC_PROD_WARPS = 8;           // epilogue warps
 constexpr int TC_THREADS = 32 * (2 + TC_PROD_WARPS);
@@ -171,6 +171,9 @@ __device__ __forceinline__ int tc_scale_exp(unsigned amax_bits) {
     const int e = (int)((amax_bits >> 23) & 0xFF);             // biased exponent
     return max(-120, min(120, 141 - e));
 }
+
+// Operand columns of a group of G maps: re and im of P values each, padded to the MMA's N.
+__host__ __device__ constexpr int tc_cols(int P, int G) { return (2 * P * G + 15) / 16 * 16; }
 
 // 32 bytes in one store (p 32-byte aligned): the 16 of two neighbouring operand rows, a whole sector.
 __device__ __forceinline__ void st_pair(char* p, const void* row0, const void* row1) {
