@@ -321,14 +321,34 @@ cudaError_t launch_legendre_adjoint_simt(const Plan& pl, const float2* ut, int B
                                          int nt, float2* out, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
     if (nt < 1 || nt > MODAL_MAXP || (!rowfilt && nt != 1)) return cudaErrorInvalidValue;
-    // the narrowest tile that holds the channels of the call, so that little work goes to padding
-    // (l_max = 1000, us for 1, 2 / 4, 8 / 16 / 32 channels: 169, 173 / 252, 254 / 418 / 715; with
-    // the 32-channel tile alone every call takes the last time)
-    const int nchan = B * nt;
-    if (nchan > 16) return legendre_adj_launch<32, 8, 4>(pl, ut, B, rowfilt, nt, out, st);
-    if (nchan > 8) return legendre_adj_launch<16, 8, 2>(pl, ut, B, rowfilt, nt, out, st);
-    if (nchan > 2) return legendre_adj_launch<8, 4, 2>(pl, ut, B, rowfilt, nt, out, st);
-    return legendre_adj_launch<2, 2, 1>(pl, ut, B, rowfilt, nt, out, st);
+    // The tile of least cost: its padded channels times its time per channel (64 channels, l_max =
+    // 400: 5.4, 2.5, 2.2 and 2.0 us), of those that give each SM 2.5 blocks; below that a narrower
+    // tile's shorter blocks are faster.  us for tiles of 2 / 8 / 16 / 32: l_max = 51, 20 channels
+    // 4.0 / 3.9 / 4.3 / 5.3; l_max = 100, 6 channels 4.3 / 4.7 / 5.7 / 7.0; l_max = 250, 11
+    // channels 22.9 / 18.6 / 17.0 / 21.6; l_max = 400, 33 channels 189 / 103 / 107 / 127.
+    // (The narrowest tile that holds all channels, up to 32, took 5.3, 4.7, 17.0 and 127.)
+    int nsm = 0;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, pl.dev);
+    // blocks of one channel tile: each order's rows of either parity in tiles of LA_BM
+    auto upto = [](int64_t n) { const int64_t q = (n + 1) / (2 * LA_BM); return LA_BM * q * (q + 1) + (n + 1) % (2 * LA_BM) * (q + 1); };
+    const int64_t rows = upto(pl.lmax) + upto(pl.lmax - 1);
+    const int width[4] = {2, 8, 16, 32}, cost_us[4] = {54, 25, 22, 20};
+    int best = -1;
+    int64_t best_cost = 0;
+    for (int i = 0; i < 4; ++i) {
+        if (width[i] < nt) continue;
+        const int cpb = rowfilt ? width[i] / nt * nt : width[i];
+        const int64_t tiles = ((int64_t)B * nt + cpb - 1) / cpb, cost = tiles * width[i] * cost_us[i];
+        if (best >= 0 && (2 * rows * tiles < 5 * nsm || cost >= best_cost)) continue;
+        best = i;
+        best_cost = cost;
+    }
+    switch (best) {
+        case 0: return legendre_adj_launch<2, 2, 1>(pl, ut, B, rowfilt, nt, out, st);
+        case 1: return legendre_adj_launch<8, 4, 2>(pl, ut, B, rowfilt, nt, out, st);
+        case 2: return legendre_adj_launch<16, 8, 2>(pl, ut, B, rowfilt, nt, out, st);
+        default: return legendre_adj_launch<32, 8, 4>(pl, ut, B, rowfilt, nt, out, st);
+    }
 }
 
 }  // namespace modal

@@ -573,8 +573,11 @@ cudaError_t launch_legendre_tc(const Plan& pl, const float2* alm, int B, float2*
     pa.L = pl.lmax;
     pa.P = pl.P;
     pa.B = B;
+    // groups of equal size, and columns for these only: with the last group padded to the full width,
+    // 12 maps of 16 modes in groups of 8 at l_max = 2000 took 13.5 ms instead of 12.8, 5 maps of 7
+    // modes at l_max = 767 457 us instead of 437
     pa.n_groups = (B + pl.tc_maps - 1) / pl.tc_maps;
-    pa.G = (B + pa.n_groups - 1) / pa.n_groups;             // groups of equal size: BALANCE
+    pa.G = (B + pa.n_groups - 1) / pa.n_groups;
     pa.N = tc_cols(pa.P, pa.G);
     pa.n_alm = pl.n_alm;
     pa.total_bkb = pl.tc.total_bkb;
