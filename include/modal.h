@@ -381,7 +381,7 @@ modal_status modal_batch_cubic(modal_batch_h bh, const void* const* alm, const i
  *     term, beta) runs chunk by chunk on its own stream, the streams concurrently.
  *   MODAL_BATCH_SHARED_CUBIC: the plans' chunks go in lockstep passes; in pass k every plan
  *     synthesizes its k-th chunk on its stream, then ONE persistent launch computes the
- *     cubic sums of all of them from a work queue of (plan, map, pixel range) items, plans
+ *     cubic sums of all of them over the list of their (plan, map, pixel range) items, plans
  *     with the longest pixel ranges first, before each plan's linear term and beta.  It
  *     applies to calls whose plans with maps share one P (at most 8 of them, at least 2);
  *     other calls run as MODAL_BATCH_STREAMS.  Every item is the one the plan's own launch

@@ -1,5 +1,5 @@
-// Plain FP32 SIMT Legendre sums (forward and transposed), one thread per ring
-// pair (forward) or per multipole l (transposed).
+// FP32 SIMT Legendre sums: forward, a register tile of modes and maps per ring pair;
+// transposed, one of multipoles l and channels.
 //
 // Forward:  D_{b,p,m}(theta) = sum_{l>=m} lambda_lm(theta) f_p(l) a_{b,lm},
 // split by the parity of l - m into E (even) and O (odd) so that one table row

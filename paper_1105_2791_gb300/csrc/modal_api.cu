@@ -1552,7 +1552,7 @@ static bool batch_shares_cubic(const modal_batch* bh, const int* B) {
 
 // Chunk passes over the plans with maps in the call.  Pass k: each plan synthesizes its k-th
 // chunk on its own stream; one persistent cubic launch on bh->main takes the (plan, map,
-// pixel range) items of every plan's chunk k from a work queue, plans with the longest pixel
+// pixel range) items of every plan's chunk k in one list, plans with the longest pixel
 // ranges first; then each plan's linear term and beta follow on its stream, and its next
 // synthesis after them.  Every item is the one the plan's own launch computes, so beta is
 // identical to modal_cubic's.
