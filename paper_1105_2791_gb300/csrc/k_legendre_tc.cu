@@ -72,17 +72,28 @@ __global__ void k_build_tc_table(int L, int R_half, int RH, int n_rt, const floa
 
 // ------------------------------------------------------------------ per-map scale
 // amax[b] = max_{l,m,p} |f_p(l) a_{b,lm}| as float bits (positive floats order as ints).
-// grid (AM_BLOCKS, B): block x takes orders m = x, x + AM_BLOCKS, ...; one atomic per warp.
+// grid (AM_BLOCKS, B): a warp takes orders m = w, w + 8 AM_BLOCKS, ..., AM_LOADS reads in flight a
+// lane, and one atomic.  us, with a block per order and one read a thread at a time, and now: 8
+// maps, l_max = 2000 70 -> 23; 12 maps, l_max = 1000 24 -> 12; 64 maps, l_max = 500 31 -> 27; 20 maps, l_max = 767 27 -> 15.
 constexpr int AM_BLOCKS = 64;
+constexpr int AM_LOADS = 8;
 __global__ void __launch_bounds__(256) k_alm_amax(int L, const float* __restrict__ fmax_l, const float2* __restrict__ alm,
                                                   int64_t n_alm, unsigned* __restrict__ amax) {
-    const int b = blockIdx.y;
+    const int b = blockIdx.y, lane = threadIdx.x & 31;
     float v = 0.f;
-    for (int m = blockIdx.x; m <= L; m += gridDim.x) {
+    for (int m = blockIdx.x * 8 + threadIdx.x / 32; m <= L; m += 8 * gridDim.x) {
         const float2* row = alm + (int64_t)b * n_alm + d_alm_index(m, m, L);
-        for (int k = threadIdx.x; k <= L - m; k += blockDim.x) {
-            const float2 a = row[k];
-            v = fmaxf(v, fmaxf(fabsf(a.x), fabsf(a.y)) * fmax_l[m + k]);
+        for (int k0 = lane; k0 <= L - m; k0 += 32 * AM_LOADS) {
+            float2 a[AM_LOADS];
+            float f[AM_LOADS];
+#pragma unroll
+            for (int i = 0; i < AM_LOADS; ++i) {
+                const int k = k0 + 32 * i;
+                a[i] = k <= L - m ? row[k] : make_float2(0.f, 0.f);
+                f[i] = k <= L - m ? fmax_l[m + k] : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < AM_LOADS; ++i) v = fmaxf(v, fmaxf(fabsf(a[i].x), fabsf(a[i].y)) * f[i]);
         }
     }
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
