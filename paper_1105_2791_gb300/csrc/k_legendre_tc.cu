@@ -405,23 +405,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_legendre_tc(TcArgs a) {
                 if (lane == 0) mbar_arrive(tmem_empty);
             };
             if (S::PRODUCTS == 3) {
-                // pairs of column blocks; TMEM is released as soon as the last pair is read
-                if (blk_hi <= blk_lo) release();
-                for (int blk = blk_lo; blk < blk_hi; blk += 2) {
-                    const bool two = blk + 1 < blk_hi;             // warp-uniform
-                    const uint32_t c0 = lane_addr + blk * 16, c1 = lane_addr + (two ? blk + 1 : blk) * 16;
+                // The last HELD blocks of the warp's columns all go to registers before any is stored:
+                // TMEM is then the next item's, whose products run beside the stores.  us with TMEM
+                // kept until the last pair was read, and now: 64 maps of 10 modes, l_max = 500 461 ->
+                // 421; 16 of 12, l_max = 1000 679 -> 643; 12 of 16, l_max = 2000 3870 -> 3692; 5 of 7,
+                // l_max = 767 (3xTF32) 280 -> 264; 16 of 12, l_max = 250 62 -> 64.  (Six blocks do
+                // not fit the 168 registers a thread has: 517, 675, 3730, 277.)
+                constexpr int HELD = 4;
+                auto load_pair = [&](int blk, bool two, float (&d0)[16], float (&d1)[16]) {
+                    const uint32_t c0 = lane_addr + blk * 16, c1 = two ? c0 + 16 : c0;
                     uint32_t r[64];
                     tmem_ld16x4(c0, c0 + N, c1, c1 + N, r);
-                    float d0[16], d1[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         d0[i] = __uint_as_float(r[i]) + __uint_as_float(r[16 + i]);
                         d1[i] = __uint_as_float(r[32 + i]) + __uint_as_float(r[48 + i]);
                     }
-                    if (blk + 2 >= blk_hi) release();
+                };
+                int blk = blk_lo;
+                for (; blk_hi - blk > HELD; blk += 2) {            // earlier blocks, a pair at a time
+                    float d0[16], d1[16];
+                    load_pair(blk, true, d0, d1);
                     store_block(blk, d0);
-                    if (two) store_block(blk + 1, d1);
+                    store_block(blk + 1, d1);
                 }
+                float d[HELD][16];
+#pragma unroll
+                for (int q = 0; q < HELD; q += 2)
+                    if (blk + q < blk_hi) load_pair(blk + q, blk + q + 1 < blk_hi, d[q], d[q + 1]);   // warp-uniform
+                release();
+#pragma unroll
+                for (int q = 0; q < HELD; ++q)
+                    if (blk + q < blk_hi) store_block(blk + q, d[q]);
             } else {
                 for (int blk = blk_lo; blk < blk_hi; ++blk) {
                     float d[16];
