@@ -89,19 +89,21 @@ cudaError_t build_pm_table(Plan& pl, cudaStream_t st) {
     }
     // the adjoint's own transforms without the filter: ring r2c of the rows W<c> (the pixel
     // weight applied as the rows are read, no ring weights), then the transposed Legendre sums
-    // of each row.  The rows go through the plan's Fourier and Legendre workspaces, as many at
-    // a time as these hold (chunk P >= n_pair in all but the smallest workspaces): neither
-    // holds anything that a later call reads, and a Legendre row of 2 (lmax + 1) RH values is
-    // longer than n_alm.
+    // of each row.  The rows go through the plan's workspace, as many at a time as it holds
+    // (chunk P >= n_pair in all but the smallest): their transforms through the adjoint's, their
+    // sums through the operand blocks of the forward Legendre sums, which take 8 bytes or more per
+    // map, mode and (l, m).  Neither outlives the call that writes it; the Legendre sums themselves
+    // (pl.delta) do, beside kept maps, and stay as they are.
     const int rows = (int)std::min<int64_t>((int64_t)pl.chunk * pl.P, pl.n_pair);
-    if (rows < 1 || !pl.ut || !pl.delta) return cudaErrorInvalidValue;
+    if (rows < 1 || !pl.ut || !pl.tc.bops) return cudaErrorInvalidValue;
+    float2* sums = static_cast<float2*>(pl.tc.bops);
     const int nlb = (pl.lmax + 32) / 32;
     for (int c0 = 0; c0 < pl.n_pair; c0 += rows) {
         const int n = std::min(rows, pl.n_pair - c0);
         cudaError_t e = launch_ring_r2c_weighted(pl, pl.pair_mean + (int64_t)c0 * pl.npix, n, pl.W, pl.ut, st);
-        if (e == cudaSuccess) e = launch_legendre_adjoint_simt(pl, pl.ut, n, nullptr, 1, pl.delta, st);
+        if (e == cudaSuccess) e = launch_legendre_adjoint_simt(pl, pl.ut, n, nullptr, 1, sums, st);
         if (e != cudaSuccess) return e;
-        k_adjpm_lmajor<<<dim3(nlb * nlb, n), 256, 0, st>>>(pl.lmax, pl.n_alm, pl.delta,
+        k_adjpm_lmajor<<<dim3(nlb * nlb, n), 256, 0, st>>>(pl.lmax, pl.n_alm, sums,
                                                            pl.adj_pm + (int64_t)c0 * pl.n_alm);
         note_launch(pl);
         e = cudaGetLastError();

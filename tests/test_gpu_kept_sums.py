@@ -1,0 +1,53 @@
+"""The Legendre sums beside kept maps: what else runs on the plan leaves them, or they are formed again, so that the
+ring-mode linear term of a retained call equals that of modal_cubic bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import simgen
+
+pytestmark = pytest.mark.gpu
+
+L, P, R, NPHI, NB = 24, 6, 25, 64, 3
+
+
+def _setup(prec, tmp_path):
+    """A plan in ring mode, its state and a pixel-mode state on files, three maps and their coefficients in ring mode."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1105_2791_gb300 as M
+    basis, cl = simgen.shifted_legendre_basis(L, P), simgen.cl_model(L)
+    make = lambda: M.Plan(L, P, basis, cl, R, NPHI, prec=prec, ring_mask=simgen.band_mask(R, 20.0))
+    sims = torch.from_numpy(simgen.gaussian_alm(cl, 6, seed=81).astype(np.complex64)).cuda()
+    a = torch.from_numpy(simgen.gaussian_alm(cl, NB, seed=82).astype(np.complex64)).cuda()
+    plan, files = make(), {}
+    for mode in ("pixel", "ring"):
+        plan.set_linear_mode(mode)
+        plan.linear_term(sims, finalize=True)
+        files[mode] = str(tmp_path / mode)
+        plan.save_state(files[mode])
+    ref = plan.cubic(a, use_linear=True)
+    plan.close()
+    return make(), files, sims, a, ref
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16x3", "3xtf32"])
+@pytest.mark.parametrize("table", ["own means", "means of earlier maps", "loaded state"])
+def test_pair_mean_table_leaves_the_kept_sums(prec, table, tmp_path):
+    """The per-pixel means' harmonic table, however it comes to be built after the maps were kept."""
+    plan, files, sims, a, ref = _setup(prec, tmp_path)
+    plan.set_retain_maps(True)
+    if table == "own means":
+        plan.linear_term(a, finalize=True)
+    elif table == "means of earlier maps":
+        plan.linear_term(sims)
+        plan.cubic(a)
+        plan.linear_term(None, finalize=True)
+    else:
+        plan.cubic(a)
+        plan.load_state(files["pixel"])
+    plan.set_linear_mode("ring")
+    plan.load_state(files["ring"])
+    assert torch.equal(plan.cubic_retained(a, use_linear=True), ref)
+    plan.sync()
+    plan.close()
