@@ -93,24 +93,33 @@ cudaError_t build_pm_table(Plan& pl, cudaStream_t st) {
     // (chunk P >= n_pair in all but the smallest): their transforms through the adjoint's, their
     // sums through the operand blocks of the forward Legendre sums, which take 8 bytes or more per
     // map, mode and (l, m).  Neither outlives the call that writes it; the Legendre sums themselves
-    // (pl.delta) do, beside kept maps, and stay as they are.
-    const int rows = (int)std::min<int64_t>((int64_t)pl.chunk * pl.P, pl.n_pair);
-    if (rows < 1 || !pl.ut || !pl.tc.bops) return cudaErrorInvalidValue;
-    float2* sums = static_cast<float2*>(pl.tc.bops);
-    const int nlb = (pl.lmax + 32) / 32;
-    for (int c0 = 0; c0 < pl.n_pair; c0 += rows) {
-        const int n = std::min(rows, pl.n_pair - c0);
-        cudaError_t e = launch_ring_r2c_weighted(pl, pl.pair_mean + (int64_t)c0 * pl.npix, n, pl.W, pl.ut, st);
-        if (e == cudaSuccess) e = launch_legendre_adjoint_simt(pl, pl.ut, n, nullptr, 1, sums, st);
+    // (pl.delta) do, beside kept maps, and stay as they are.  A plan that a failed modal_set_chunk
+    // left without workspace (modal_load_state still fills its means) takes temporaries for the
+    // rows of one map.
+    const size_t row = (size_t)(pl.lmax + 1) * 2 * pl.RH;
+    const bool own = pl.chunk < 1;
+    const int rows = (int)std::min<int64_t>((int64_t)(own ? 1 : pl.chunk) * pl.P, pl.n_pair);
+    float2 *ut = pl.ut, *sums = static_cast<float2*>(pl.tc.bops);
+    if (own) {
+        const cudaError_t e = cudaMallocAsync(&ut, rows * (row + pl.n_alm) * sizeof(float2), st);
         if (e != cudaSuccess) return e;
+        sums = ut + rows * row;
+    }
+    const int nlb = (pl.lmax + 32) / 32;
+    cudaError_t e = cudaSuccess;
+    for (int c0 = 0; e == cudaSuccess && c0 < pl.n_pair; c0 += rows) {
+        const int n = std::min(rows, pl.n_pair - c0);
+        e = launch_ring_r2c_weighted(pl, pl.pair_mean + (int64_t)c0 * pl.npix, n, pl.W, ut, st);
+        if (e == cudaSuccess) e = launch_legendre_adjoint_simt(pl, ut, n, nullptr, 1, sums, st);
+        if (e != cudaSuccess) break;
         k_adjpm_lmajor<<<dim3(nlb * nlb, n), 256, 0, st>>>(pl.lmax, pl.n_alm, sums,
                                                            pl.adj_pm + (int64_t)c0 * pl.n_alm);
         note_launch(pl);
         e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
     }
-    pl.adj_pm_ready = 1;
-    return cudaSuccess;
+    if (own) cudaFreeAsync(ut, st);
+    if (e == cudaSuccess) pl.adj_pm_ready = 1;
+    return e;
 }
 
 // K[l][b][c] = sum_t f_t(l) h_{b,t,c}
