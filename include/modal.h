@@ -36,7 +36,8 @@
  *  - A plan is not thread-safe; calls on one plan whose work overlaps on the
  *    GPU (different streams) race, with one exception: the FP64 solve family
  *    (modal_solve, modal_fnl_weights) reads only the covariance sums and its
- *    arguments and writes only its own stream-ordered workspace and its own
+ *    arguments and writes only its own workspace (the plan's, kept between such
+ *    calls, each of which has ended on the GPU when it returns) and its own
  *    device error word, so it may run on a second stream beside modal_backward
  *    or modal_backward_retained of the same plan, issued from the same host
  *    thread, once the covariance sums it reads are complete on its stream (an

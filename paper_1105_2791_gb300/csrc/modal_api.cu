@@ -933,8 +933,9 @@ static modal_status read_device_error(modal_h h, cudaStream_t st, int* word) {
 
 // The FP64 workspace of one modal_solve or modal_fnl_weights call: zeta and its factor, the
 // carried rows (alpha, betas), the diagonal-block scratch and the results with the error word.
-// Up to kSolveKeep carried rows it is the plan's own, allocated by the first such call (both
-// calls synchronise, so one plan never needs two); a larger batch allocates for the call.
+// Up to kSolveKeep carried rows it is the plan's own, allocated by the first such call and kept (both
+// calls have ended on the GPU when they return, whatever their status, so one plan never needs
+// two); a larger batch allocates for the call.
 constexpr int kSolveKeep = 257;
 
 struct SolveSpace {
@@ -961,10 +962,12 @@ static modal_status solve_space(modal_h h, int nrows, cudaStream_t st, SolveSpac
     return MODAL_OK;
 }
 
-static void release(SolveSpace& sp, cudaStream_t st) {
-    if (!sp.owned) return;
-    cudaFreeAsync(sp.owned, st);
-    cudaStreamSynchronize(st);
+// After a call that ended in status s: a temporary goes back, and nothing of a failed call (a success
+// has waited for its results) still runs in the plan's workspace when the next one starts.
+static modal_status release(SolveSpace& sp, modal_status s, cudaStream_t st) {
+    if (sp.owned) cudaFreeAsync(sp.owned, st);
+    if (sp.owned || s != MODAL_OK) cudaStreamSynchronize(st);
+    return s;
 }
 
 // The error word that came back with the results of a solve (out[count]); clears it.
@@ -996,7 +999,7 @@ modal_status modal_fnl_weights(modal_h h, const double* alpha, double* w, double
     if (h->n_cov < 2) return set_error(MODAL_ESTATE, "need at least 2 covariance simulations");
     cudaStream_t st = as_stream(stream);
     SolveSpace sp;
-    modal_status s = solve_space(h, 1, st, &sp);
+    const modal_status s = solve_space(h, 1, st, &sp);
     if (s != MODAL_OK) return s;
     auto run = [&]() -> modal_status {
         const modal_status f = factor_with_rows(h, sp, alpha, nullptr, 0, st);
@@ -1011,9 +1014,7 @@ modal_status modal_fnl_weights(modal_h h, const double* alpha, double* w, double
         if (sigma) *sigma = std::sqrt(6.0 / out[0]);
         return MODAL_OK;
     };
-    s = run();
-    release(sp, st);
-    return s;
+    return release(sp, run(), st);
 }
 
 modal_status modal_solve(modal_h h, const double* alpha, const double* beta, int B, double* fnl, double* sigma,
@@ -1023,7 +1024,7 @@ modal_status modal_solve(modal_h h, const double* alpha, const double* beta, int
     if (h->n_cov < 2) return set_error(MODAL_ESTATE, "need at least 2 covariance simulations");
     cudaStream_t st = as_stream(stream);
     SolveSpace sp;
-    modal_status s = solve_space(h, B + 1, st, &sp);
+    const modal_status s = solve_space(h, B + 1, st, &sp);
     if (s != MODAL_OK) return s;
     auto run = [&]() -> modal_status {
         const modal_status f = factor_with_rows(h, sp, alpha, beta, B, st);
@@ -1038,9 +1039,7 @@ modal_status modal_solve(modal_h h, const double* alpha, const double* beta, int
         for (int b = 0; b < B; ++b) fnl[b] = out[1 + b];
         return MODAL_OK;
     };
-    s = run();
-    release(sp, st);
-    return s;
+    return release(sp, run(), st);
 }
 
 // Power iteration of the bivector fit: stop when |Z v - lam v| <= kPowerTol |lam|, checked

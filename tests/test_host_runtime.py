@@ -65,3 +65,24 @@ def test_state_loads_into_a_plan_without_workspace(lib, prec, tmp_path):
     B.modal_set_chunk(h, 2)
     B.modal_cubic(h, buf.ctypes.data, 1, True, buf.ctypes.data, stream=0)
     B.modal_destroy(h)
+
+
+@pytest.mark.parametrize("maps", [2, 300])                  # the plan's own workspace; one allocated for the call
+@pytest.mark.parametrize("call,copies", [("solve", 3), ("weights", 2)])
+def test_failed_solve_leaves_nothing_running(lib, call, copies, maps):
+    """Whichever copy of a solve fails, what it queued before has ended when the error is returned: the next call, on any
+    stream, may use the same workspace."""
+    h = _plan("fp32")
+    n = B.modal_get_info(h).n_max
+    buf = np.zeros(1 << 16)
+    B.modal_cov_accumulate(h, buf.ctypes.data, 3, stream=0)
+    for k in range(1, copies + 1):
+        lib.fake_fail_copy(k)
+        with pytest.raises(B.ModalError) as e:
+            if call == "solve":
+                B.modal_solve(h, np.ones(n), buf.ctypes.data, maps, stream=0)
+            else:
+                B.modal_fnl_weights(h, np.ones(n), buf.ctypes.data, stream=0)
+        assert e.value.status == B.MODAL_ECUDA
+        assert lib.fake_pending() == 0 and lib.fake_live() == 0
+    B.modal_destroy(h)
