@@ -379,22 +379,29 @@ static CubicShape cubic_shape(const Plan& pl) {
     return sh;
 }
 
-static CubicJob cubic_job(const Plan& pl, int B, double* partial) {
+static int64_t cubic_ppc(const Plan& pl) { return ((pl.npix + pl.cubic_ctas - 1) / pl.cubic_ctas + CUB_TX - 1) / CUB_TX * CUB_TX; }
+
+// The tiled copies take 32-bit pixel coordinates, which run to one range past the map's end.
+constexpr int64_t CUB_COORDS = (int64_t)1 << 31;
+bool cubic_one_launch(const Plan& pl) { return pl.npix + cubic_ppc(pl) < CUB_COORDS; }
+
+// B maps, their first `npix` pixels in `nctas` ranges
+static CubicJob cubic_job(const Plan& pl, int B, int64_t npix, int nctas, double* partial) {
     CubicJob jb;
     jb.partial = partial;
-    jb.npix = pl.npix;
-    jb.ppc = ((pl.npix + pl.cubic_ctas - 1) / pl.cubic_ctas + CUB_TX - 1) / CUB_TX * CUB_TX;
-    jb.nctas = pl.cubic_ctas;
-    jb.nunits = (int64_t)B * pl.cubic_ctas;
+    jb.npix = npix;
+    jb.ppc = cubic_ppc(pl);
+    jb.nctas = nctas;
+    jb.nunits = (int64_t)B * nctas;
     return jb;
 }
 
-static cudaError_t cubic_tiles(const Plan& pl, const float* maps, int B, CubicTiles* tl) {
-    const cuuint64_t dims[2] = {(cuuint64_t)pl.npix, (cuuint64_t)B * pl.P}, wdims[2] = {(cuuint64_t)pl.npix, 1};
+static cudaError_t cubic_tiles(const Plan& pl, const float* maps, const float* W, int B, int64_t npix, CubicTiles* tl) {
+    const cuuint64_t dims[2] = {(cuuint64_t)npix, (cuuint64_t)B * pl.P}, wdims[2] = {(cuuint64_t)npix, 1};
     const cuuint64_t strides[1] = {(cuuint64_t)pl.npix * sizeof(float)};
     const cuuint32_t box[2] = {CUB_ROW, (cuuint32_t)pl.P}, wbox[2] = {CUB_ROW, 1};
     const cudaError_t e = tma_map_f32(&tl->maps, maps, 2, dims, strides, box);
-    return e != cudaSuccess ? e : tma_map_f32(&tl->W, pl.W, 2, wdims, strides, wbox);
+    return e != cudaSuccess ? e : tma_map_f32(&tl->W, W, 2, wdims, strides, wbox);
 }
 
 cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, const int* B, int n, cudaStream_t st) {
@@ -405,9 +412,9 @@ cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, con
     int64_t total = 0;
     for (int i = 0; i < n; ++i) {
         const Plan& pl = *plans[i];
-        if (pl.P != p0.P || B[i] < 1 || B[i] > pl.chunk) return cudaErrorInvalidValue;
-        jobs.job[i] = cubic_job(pl, B[i], pl.partial);
-        const cudaError_t e = cubic_tiles(pl, maps[i], B[i], &jobs.tiles[i]);
+        if (pl.P != p0.P || B[i] < 1 || B[i] > pl.chunk || !cubic_one_launch(pl)) return cudaErrorInvalidValue;
+        jobs.job[i] = cubic_job(pl, B[i], pl.npix, pl.cubic_ctas, pl.partial);
+        const cudaError_t e = cubic_tiles(pl, maps[i], pl.W, B[i], pl.npix, &jobs.tiles[i]);
         if (e != cudaSuccess) return e;
         total += (jobs.job[i].nunits + 1) / 2 * sh.ngroups;
         jobs.item_end[i] = total;
@@ -424,21 +431,41 @@ cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st) {
-    if (B == 0) return cudaSuccess;
+static cudaError_t cubic_launch(const Plan& pl, const CubicTiles& tl, const CubicJob& jb, cudaStream_t st) {
     const CubicShape sh = cubic_shape(pl);
-    const CubicJob jb = cubic_job(pl, B, partial);
-    CubicTiles tl;
-    cudaError_t e = cubic_tiles(pl, maps, B, &tl);
-    if (e != cudaSuccess) return e;
     const size_t smem = cubic_smem(sh);
     auto kernel = cubic_half(pl.P) ? k_cubic<true> : k_cubic<false>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t items = (jb.nunits + 1) / 2 * sh.ngroups;
     kernel<<<(unsigned)items, (sh.nbox + 1) * 32, smem, st>>>(tl, jb, sh, pl.d_err);
     note_launch(pl);
     return cudaGetLastError();
+}
+
+cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st) {
+    if (B == 0) return cudaSuccess;
+    CubicTiles tl;
+    if (cubic_one_launch(pl)) {
+        const cudaError_t e = cubic_tiles(pl, maps, pl.W, B, pl.npix, &tl);
+        return e != cudaSuccess ? e : cubic_launch(pl, tl, cubic_job(pl, B, pl.npix, pl.cubic_ctas, partial), st);
+    }
+    // larger maps one by one, as many whole ranges at a time as the coordinates reach; ranges past
+    // the last pixel (their sums are zero) go with the last part
+    const int64_t ppc = cubic_ppc(pl);
+    const int per = (int)((CUB_COORDS - 1) / ppc) - 1, full = (int)((pl.npix + ppc - 1) / ppc);
+    if (per < 1) return cudaErrorInvalidValue;
+    for (int b = 0; b < B; ++b)
+        for (int r0 = 0; r0 < full; r0 += per) {
+            const bool last = r0 + per >= full;
+            const int64_t x0 = r0 * ppc, n = last ? pl.npix - x0 : per * ppc;
+            cudaError_t e = cubic_tiles(pl, maps + (int64_t)b * pl.P * pl.npix + x0, pl.W + x0, 1, n, &tl);
+            if (e == cudaSuccess)
+                e = cubic_launch(pl, tl, cubic_job(pl, 1, n, last ? pl.cubic_ctas - r0 : per,
+                                                   partial + ((int64_t)b * pl.cubic_ctas + r0) * pl.n_max), st);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 // ---------------------------------------------------------------- linear term GEMM

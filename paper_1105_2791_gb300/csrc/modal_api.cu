@@ -1533,7 +1533,8 @@ static void batch_drop_graph(modal_batch* bh) {
 }
 
 // True if the plans' cubic sums can share one launch: the same P (so the same mode tables
-// and kernel instance) and at most CUBIC_MAX_JOBS plans with maps in the call.
+// and kernel instance), maps that one launch can address and at most CUBIC_MAX_JOBS plans with
+// maps in the call.
 static bool batch_shares_cubic(const modal_batch* bh, const int* B) {
     if (bh->schedule != MODAL_BATCH_SHARED_CUBIC) return false;
     int n = 0;
@@ -1542,8 +1543,7 @@ static bool batch_shares_cubic(const modal_batch* bh, const int* B) {
         if (B[i] == 0) continue;
         const modal_plan* p = bh->plans[i];
         if (!p0) p0 = p;
-        if (p->P != p0->P || p->n_max != p0->n_max)
-            return false;
+        if (p->P != p0->P || p->n_max != p0->n_max || !cubic_one_launch(*p)) return false;
         ++n;
     }
     return n >= 2 && n <= CUBIC_MAX_JOBS;

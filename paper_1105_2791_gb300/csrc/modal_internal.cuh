@@ -219,6 +219,7 @@ cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cu
 // buffer) of n plans with the same P as one persistent launch.
 constexpr int CUBIC_MAX_JOBS = 8;
 constexpr int CUBIC_BOXES = 10;      // warps per CTA of the cubic kernel, one box each
+bool cubic_one_launch(const Plan& pl);   // false from nearly 2^31 pixels: then only launch_cubic, in parts
 cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, const int* B, int n, cudaStream_t st);
 cudaError_t launch_linear_gemm(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st);
 // lin_splits: K splits summed from lin_partial ([lin_splits][n_pair][B P])

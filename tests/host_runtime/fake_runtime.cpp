@@ -8,6 +8,9 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <vector>
+
+#include "modal_internal.cuh"
 
 
 namespace {
@@ -15,8 +18,22 @@ std::map<const void*, std::string> names;   // host stub -> kernel
 int fail_alloc = 0, fail_copy = 0;           // every allocation; the fail_copy-th asynchronous copy from now
 long long pending = 0, live = 0;             // operations queued since the last wait; temporaries held
 void queued() { ++pending; }
-CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill) {
+dim3 launch_grid;
+struct Tiles {                               // an encoded tensor map of two dimensions
+    long long base, cols, rows, pitch;
+};
+std::vector<Tiles> encoded;
+struct Job {                                 // the second argument of k_cubic
+    double* partial;
+    int64_t npix, ppc;
+    int nctas;
+    int64_t nunits;
+};
+std::vector<long long> cubic_log;            // per launch of k_cubic: its two tensor maps and its job
+CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+                CUtensorMapFloatOOBfill) {
+    if (rank == 2) encoded.push_back({(long long)base, (long long)dims[0], (long long)dims[1], (long long)strides[0]});
     return CUDA_SUCCESS;
 }
 cudaError_t allocate(void** p, size_t n) {
@@ -33,6 +50,22 @@ void fake_fail_alloc(int on) { fail_alloc = on; }
 void fake_fail_copy(int nth) { fail_copy = nth; }
 long long fake_pending() { return pending; }
 long long fake_live() { return live; }
+// The launches of the cubic sums of B maps at address `maps` (weights W, partial sums at `partial`): twelve values each into out.
+int fake_cubic(long long npix, int P, int B, int ctas, long long maps, long long W, long long partial, long long* out, int max) {
+    modal::Plan pl;
+    pl.P = P;
+    pl.npix = npix;
+    pl.n_max = P * (P + 1) * (P + 2) / 6;
+    pl.cubic_ctas = ctas;
+    pl.cubic_groups = 1;
+    pl.cubic_boxes = 1;
+    pl.nsm = 152;
+    pl.W = reinterpret_cast<float*>(W);
+    cubic_log.clear();
+    if (modal::launch_cubic(pl, reinterpret_cast<const float*>(maps), B, reinterpret_cast<double*>(partial), nullptr) != cudaSuccess) return -1;
+    for (size_t i = 0; i < cubic_log.size() && i < (size_t)max; ++i) out[i] = cubic_log[i];
+    return (int)cubic_log.size() / 12;
+}
 
 // registration and launches
 void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
@@ -40,10 +73,20 @@ void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) { names[host] = name; }
-unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, cudaStream_t) { return 0; }
-cudaError_t __cudaPopCallConfiguration(dim3*, dim3*, size_t*, void*) { return cudaSuccess; }
+unsigned __cudaPushCallConfiguration(dim3 grid, dim3, size_t, cudaStream_t) { launch_grid = grid; return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3* grid, dim3*, size_t*, void*) { *grid = launch_grid; return cudaSuccess; }
 cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* host) { *k = (cudaKernel_t)host; return cudaSuccess; }
-cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void**, size_t, cudaStream_t) { queued(); return cudaSuccess; }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void** args, size_t, cudaStream_t) {
+    queued();
+    if (names[k].find("7k_cubicILb") != std::string::npos && encoded.size() >= 2) {
+        const Tiles &m = encoded[encoded.size() - 2], &w = encoded.back();
+        const Job& j = *static_cast<const Job*>(args[1]);
+        for (long long v : {m.base, m.cols, m.rows, m.pitch, w.base, w.cols, (long long)j.partial, (long long)j.npix, (long long)j.ppc,
+                            (long long)j.nctas, (long long)j.nunits, (long long)grid.x})
+            cubic_log.push_back(v);
+    }
+    return cudaSuccess;
+}
 
 cudaError_t cudaMalloc(void** p, size_t n) { return allocate(p, n); }
 cudaError_t cudaFree(void* p) { std::free(p); return cudaSuccess; }

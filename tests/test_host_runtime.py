@@ -86,3 +86,33 @@ def test_failed_solve_leaves_nothing_running(lib, call, copies, maps):
         assert e.value.status == B.MODAL_ECUDA
         assert lib.fake_pending() == 0 and lib.fake_live() == 0
     B.modal_destroy(h)
+
+
+# the last size of one launch, one past it, 2^31 pixels, and far more than 2^32 in several parts per map
+@pytest.mark.parametrize("npix,ctas", [(1 << 20, 128), ((1 << 31) - 16, 152), (1 << 31, 152), (300000 * 8192, 152), (9 << 31, 152), (3 << 29, 2)])
+@pytest.mark.parametrize("maps,P", [(1, 3), (3, 2)])
+def test_cubic_launches_cover_maps_of_any_size(lib, npix, ctas, maps, P):
+    """The tiled copies take 32-bit pixel coordinates: whatever the number of pixels, each pixel range of each map is
+    one launch's, at the addresses and with the partial sums of the whole, and no coordinate reaches 2^31."""
+    A, W, S, n_max = 1 << 40, 1 << 50, 1 << 56, P * (P + 1) * (P + 2) // 6
+    out = (ctypes.c_longlong * 12000)()
+    lib.fake_cubic.argtypes = [ctypes.c_longlong] + [ctypes.c_int] * 3 + [ctypes.c_longlong] * 3 + [ctypes.c_void_p, ctypes.c_int]
+    n = lib.fake_cubic(npix, P, maps, ctas, A, W, S, out, len(out))
+    assert 1 <= n <= 1000
+    whole = (-(-npix // ctas) + 127) // 128 * 128           # pixels of a range
+    seen = set()
+    for k in range(n):
+        base, cols, rows, pitch, wbase, wcols, partial, px, ppc, nctas, nunits, grid = out[12 * k:12 * k + 12]
+        assert ppc == whole and pitch == 4 * npix and cols == wcols == px and rows == P * (nunits // nctas)
+        assert px + ppc < 1 << 31 and nunits % nctas == 0 and grid == (nunits + 1) // 2
+        for u in range(nunits):
+            slot = (partial - S) // 8 // n_max + u
+            b, r = divmod(slot, ctas)
+            at = u // nctas * P * npix * 4 + u % nctas * ppc * 4   # where the launch reads unit u, from its maps
+            if r * whole < npix:
+                assert base + at == A + (b * P * npix + r * whole) * 4
+                assert wbase + u % nctas * ppc * 4 == W + r * whole * 4
+                assert min(px, (u % nctas + 1) * ppc) - u % nctas * ppc == min(npix, (r + 1) * whole) - r * whole
+            assert slot not in seen
+            seen.add(slot)
+    assert seen == set(range(maps * ctas))
