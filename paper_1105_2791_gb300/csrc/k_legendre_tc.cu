@@ -245,7 +245,10 @@ __device__ __forceinline__ void tc_item(const TcArgs& a, int64_t item, int& m, i
     m = (int)(t >> 1);
 }
 
-template <int PREC>
+// HELD: how many of an epilogue warp's last column blocks go to registers before any of them is
+// stored (0: a loop over pairs of blocks, nothing held past a pair).  TMEM is then the next item's,
+// whose products run beside the stores; before that the stores wait for the reads (tc_held).
+template <int PREC, int HELD>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_legendre_tc(TcArgs a) {
     using S = Split<PREC>;
     constexpr bool TF32 = (PREC == MODAL_3XTF32);
@@ -405,13 +408,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_legendre_tc(TcArgs a) {
                 if (lane == 0) mbar_arrive(tmem_empty);
             };
             if (S::PRODUCTS == 3) {
-                // The last HELD blocks of the warp's columns all go to registers before any is stored:
-                // TMEM is then the next item's, whose products run beside the stores.  us with TMEM
-                // kept until the last pair was read, and now: 64 maps of 10 modes, l_max = 500 461 ->
-                // 421; 16 of 12, l_max = 1000 679 -> 643; 12 of 16, l_max = 2000 3870 -> 3692; 5 of 7,
-                // l_max = 767 (3xTF32) 280 -> 264; 16 of 12, l_max = 250 62 -> 64.  (Six blocks do
-                // not fit the 168 registers a thread has: 517, 675, 3730, 277.)
-                constexpr int HELD = 4;
                 auto load_pair = [&](int blk, bool two, float (&d0)[16], float (&d1)[16]) {
                     const uint32_t c0 = lane_addr + blk * 16, c1 = two ? c0 + 16 : c0;
                     uint32_t r[64];
@@ -422,21 +418,33 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_legendre_tc(TcArgs a) {
                         d1[i] = __uint_as_float(r[32 + i]) + __uint_as_float(r[48 + i]);
                     }
                 };
-                int blk = blk_lo;
-                for (; blk_hi - blk > HELD; blk += 2) {            // earlier blocks, a pair at a time
-                    float d0[16], d1[16];
-                    load_pair(blk, true, d0, d1);
-                    store_block(blk, d0);
-                    store_block(blk + 1, d1);
+                if constexpr (HELD == 0) {
+                    if (blk_hi <= blk_lo) release();
+                    for (int blk = blk_lo; blk < blk_hi; blk += 2) {
+                        const bool two = blk + 1 < blk_hi;         // warp-uniform
+                        float d0[16], d1[16];
+                        load_pair(blk, two, d0, d1);
+                        if (blk + 2 >= blk_hi) release();
+                        store_block(blk, d0);
+                        if (two) store_block(blk + 1, d1);
+                    }
+                } else {
+                    int blk = blk_lo;
+                    for (; blk_hi - blk > HELD; blk += 2) {        // earlier blocks, a pair at a time
+                        float d0[16], d1[16];
+                        load_pair(blk, true, d0, d1);
+                        store_block(blk, d0);
+                        store_block(blk + 1, d1);
+                    }
+                    float d[HELD][16];
+#pragma unroll
+                    for (int q = 0; q < HELD; q += 2)
+                        if (blk + q < blk_hi) load_pair(blk + q, blk + q + 1 < blk_hi, d[q], d[q + 1]);   // warp-uniform
+                    release();
+#pragma unroll
+                    for (int q = 0; q < HELD; ++q)
+                        if (blk + q < blk_hi) store_block(blk + q, d[q]);
                 }
-                float d[HELD][16];
-#pragma unroll
-                for (int q = 0; q < HELD; q += 2)
-                    if (blk + q < blk_hi) load_pair(blk + q, blk + q + 1 < blk_hi, d[q], d[q + 1]);   // warp-uniform
-                release();
-#pragma unroll
-                for (int q = 0; q < HELD; ++q)
-                    if (blk + q < blk_hi) store_block(blk + q, d[q]);
             } else {
                 for (int blk = blk_lo; blk < blk_hi; ++blk) {
                     float d[16];
@@ -562,6 +570,21 @@ void free_tc_tables(Plan& pl) {
     pl.tc = TcTable();
 }
 
+// Column blocks to hold (k_legendre_tc): nothing to choose up to two per warp; four where an item has
+// K blocks enough (nkb: the longest item's) for its products to outlast the later start of the
+// stores, else two.  The line lies at eight, at six where three blocks are all the warp has.  us with
+// 0 / 2 / 4 held, FP16x3: l_max = 300 (nkb 5), 32 maps of 3, 7, 12 and 16 modes 67 / 70 / 72, 101 / 100 /
+// 106, 141 / 135 / 143 and 180 / 170 / 178; l_max = 420 (7), 6 and 12 modes 142 / 137 / 133 and 211 /
+// 203 / 206; l_max = 600 (10) 335 / 325 / 303 and 472 / 456 / 443; l_max = 1000, 7 and 16 modes 975 / 962
+// / 911 and 1577 / 1513 / 1507; 12 maps of 16 modes, l_max = 2000 3859 / 3783 / 3668.  3xTF32, 16 maps:
+// l_max = 125 (4), 12 modes 24.5 / 24.5 / 25.8; l_max = 500 (16) 197 / 193 / 188.  (Six held do not fit
+// the 168 registers a thread has.)
+static int tc_held(int N, int nkb) {
+    const int blocks = (N / 16 + 1) / 2;
+    if (blocks <= 2) return 0;
+    return nkb >= (blocks == 3 ? 6 : 8) ? 4 : 2;
+}
+
 template <int PREC>
 static cudaError_t launch_tc(const Plan& pl, const PrepArgs& pa, const TcArgs& args, int part, cudaStream_t st) {
     if (part & 1) {
@@ -573,15 +596,26 @@ static cudaError_t launch_tc(const Plan& pl, const PrepArgs& pa, const TcArgs& a
         if (e != cudaSuccess) return e;
     }
     if (!(part & 2)) return cudaSuccess;
-    const size_t smem = tc_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(k_legendre_tc<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int nsm = 0;
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, pl.dev);
-    const int grid = (int)std::min<int64_t>(args.n_items, (int64_t)std::max(nsm, 1));
-    k_legendre_tc<PREC><<<grid, TC_THREADS, smem, st>>>(args);
-    note_launch(pl);
-    return cudaGetLastError();
+    auto run = [&](auto held) -> cudaError_t {
+        auto kernel = k_legendre_tc<PREC, decltype(held)::value>;
+        const size_t smem = tc_smem_bytes();
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        int nsm = 0;
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, pl.dev);
+        const int grid = (int)std::min<int64_t>(args.n_items, (int64_t)std::max(nsm, 1));
+        kernel<<<grid, TC_THREADS, smem, st>>>(args);
+        note_launch(pl);
+        return cudaGetLastError();
+    };
+    if constexpr (Split<PREC>::PRODUCTS == 3) {
+        switch (tc_held(args.N, tc_nkb(pl.lmax, 0, 0, kps_for(pl.prec)))) {
+            case 4: return run(std::integral_constant<int, 4>());
+            case 2: return run(std::integral_constant<int, 2>());
+            default: break;
+        }
+    }
+    return run(std::integral_constant<int, 0>());
 }
 
 cudaError_t launch_legendre_tc(const Plan& pl, const float2* alm, int B, float2* delta, int part, cudaStream_t st) {
