@@ -260,7 +260,7 @@ constexpr int CUB_THREADS = (CUBIC_BOXES + 1) * 32;
 // of modes holds at most two.  The warps of a CTA run as many different box bodies as there are
 // shapes, so the instruction cache decides how far the pixel loop is unrolled: with four shapes
 // all 8 pixels of a stage (16 modes, l_max = 1000, 16 maps: 1.51 ms, 1.63 looped), with the
-// eight that a half block brings two at a time (10 modes, l_max = 500, 64 maps: 0.72 ms looped,
+// eight that a half block brings (up to 10 modes: cubic_half) two at a time (10 modes, l_max = 500, 64 maps: 0.72 ms looped,
 // 1.05 unrolled, 0.91 with the last block treated as whole).
 template <bool HALF>
 struct CubicCta {
@@ -363,9 +363,6 @@ static size_t cubic_smem(const CubicShape& sh) {
     const size_t red = (size_t)2 * sh.nbox * CUB_LANES * CUB_RED;
     return (stages + red) * sizeof(float) + 128;
 }
-
-// whether the boxes have half blocks (as the plan built them)
-static bool cubic_half(int P) { return P % 4 == 1 || P % 4 == 2; }
 
 static CubicShape cubic_shape(const Plan& pl) {
     CubicShape sh;

@@ -122,7 +122,7 @@ static void build_mode_tables(modal_plan* pl, std::vector<int>& prs, std::vector
 // sub-partitions out (the sum of squares falls).
 static void build_cubic_boxes(modal_plan* pl, std::vector<int>& boxes) {
     const int nb = (pl->P + 3) / 4;
-    const bool half = pl->P % 4 == 1 || pl->P % 4 == 2;      // the last block holds at most two modes
+    const bool half = cubic_half(pl->P);                     // the last block holds at most two modes
     // packed multiply-adds per pixel, pair products included, by shape and half
     auto weight = [](int code) {
         static const int w[2][4] = {{42, 32, 30, 21}, {26, 20, 12, 6}};

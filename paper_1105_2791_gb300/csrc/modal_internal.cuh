@@ -219,6 +219,11 @@ cudaError_t launch_cubic(Plan& pl, const float* maps, int B, double* partial, cu
 // buffer) of n plans with the same P as one persistent launch.
 constexpr int CUBIC_MAX_JOBS = 8;
 constexpr int CUBIC_BOXES = 10;      // warps per CTA of the cubic kernel, one box each
+// Whether a last block of at most two modes has box shapes of its own (as the plan builds its boxes):
+// up to 10 modes, whose boxes are one group.  At 13 and 14 modes the two CTAs of a pair of units
+// would each run up to eight box bodies, whose instructions do not stay cached: 128 ranges of
+// 8192 pixels 94 us, and as four whole blocks, the operations of the kept sums the same, 65 (90 and 92 as pair-product panels).
+inline bool cubic_half(int P) { return P <= 10 && (P % 4 == 1 || P % 4 == 2); }
 bool cubic_one_launch(const Plan& pl);   // false from nearly 2^31 pixels: then only launch_cubic, in parts
 cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, const int* B, int n, cudaStream_t st);
 cudaError_t launch_linear_gemm(Plan& pl, const float* maps, int B, double* partial, cudaStream_t st);
