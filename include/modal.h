@@ -218,7 +218,8 @@ modal_status modal_set_retain_maps(modal_h h, int on);
 
 /* modal_cubic (Eq. bbispect with the linear term of Eq. bispectrumest) at the a_lm of the
  * plan's last modal_linear_term or modal_cubic call, from the maps that call kept (and, for
- * the per-ring linear term, the Legendre sums still beside them): the same result as
+ * the per-ring linear term, the Legendre sums beside them, formed again from the a_lm if
+ * modal_synthesize has run on the plan since): the same result as
  * modal_cubic(h, alm, B, use_linear, beta) without the synthesis, so that a batch that is
  * both a linear-term sample and a coefficient input is synthesised once.  alm and B must
  * be the pointer and count given to that call (checked; the caller must not have changed

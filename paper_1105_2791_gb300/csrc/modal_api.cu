@@ -340,6 +340,7 @@ static cudaError_t legendre_forward(modal_plan* pl, const float2* alm, int B, cu
 
 static cudaError_t synth_chunk(modal_plan* pl, const float2* alm, int B, float* maps_out, cudaStream_t st) {
     if (maps_out == pl->maps) pl->kept_alm = nullptr;
+    pl->kept_sums = 0;
     {
         cudaError_t e = legendre_forward(pl, alm, B, st);
         if (e != cudaSuccess) return e;
@@ -740,6 +741,14 @@ static modal_status refresh_pm_table(modal_plan* h, cudaStream_t st) {
     return MODAL_OK;
 }
 
+static void keep_maps_if_whole(modal_h h, const void* alm, int B) {
+    if (h->retain_maps && B > 0 && B <= h->chunk) {      // the whole batch is in the map workspace
+        h->kept_alm = alm;
+        h->kept_B = B;
+        h->kept_sums = 1;
+    }
+}
+
 modal_status modal_linear_term(modal_h h, const void* alm_sims, int B, int finalize, void* stream) {
     if (check_plan(h)) return MODAL_EINVAL;
     if (check_workspace(h)) return MODAL_ESTATE;
@@ -758,10 +767,7 @@ modal_status modal_linear_term(modal_h h, const void* alm_sims, int B, int final
         else CK(launch_pair_accumulate(*h, h->maps, nb, st), "pair accumulate");
     }
     h->n_lin += B;
-    if (h->retain_maps && B > 0 && B <= h->chunk) {      // the whole batch is in the map workspace
-        h->kept_alm = alm_sims;
-        h->kept_B = B;
-    }
+    keep_maps_if_whole(h, alm_sims, B);
     if (finalize) {
         if (h->n_lin < 1) return set_error(MODAL_ESTATE, "finalize with no linear-term simulations");
         STAGE(h, ST_PAIRS, st);
@@ -812,24 +818,21 @@ static modal_status cubic_chunk_tail(modal_h h, const float2* a, int nb, int use
     return MODAL_OK;
 }
 
-static void keep_maps_if_whole(modal_h h, const void* alm, int B) {
-    if (h->retain_maps && B > 0 && B <= h->chunk) {      // the whole batch is in the map workspace
-        h->kept_alm = alm;
-        h->kept_B = B;
-    }
-}
-
 static modal_status cubic_impl(modal_h h, const void* alm, int B, int use_linear, double* beta, cudaStream_t st,
                                bool kept) {
     const float2* a = static_cast<const float2*>(alm);
     for (int b0 = 0; b0 < B; b0 += h->chunk) {
         const int nb = std::min(h->chunk, B - b0);
         if (!kept) CK(synth_chunk(h, a + (size_t)b0 * h->n_alm, nb, h->maps, st), "cubic synthesis");
+        else if (use_linear && h->lin_mode == MODAL_LINEAR_RING && !h->kept_sums) {
+            CK(legendre_forward(h, a, nb, st), "Legendre sums of kept maps");    // overwritten since by modal_synthesize
+            h->kept_sums = 1;
+        }
         { STAGE(h, ST_CUBIC, st); CK(launch_cubic(*h, h->maps, nb, h->partial, st), "cubic"); }
         const modal_status r = cubic_chunk_tail(h, a + (size_t)b0 * h->n_alm, nb, use_linear, beta + (size_t)b0 * h->n_max, st);
         if (r != MODAL_OK) return r;
     }
-    keep_maps_if_whole(h, alm, B);
+    if (!kept) keep_maps_if_whole(h, alm, B);
     return MODAL_OK;
 }
 

@@ -136,6 +136,7 @@ struct Plan {
     int retain_maps = 0;
     const void* kept_alm = nullptr;   // a_lm they were synthesised from (nullptr: none kept)
     int kept_B = 0;
+    int kept_sums = 0;                // their Legendre sums are still in `delta`
     float* hk = nullptr;         // [chunk][P][n_pair] adjoint weights
     char* adj_gops = nullptr;    // [chunk] tf32 hi/lo G operands of the tensor-core adjoint pixel weights
     float* adj_pmk = nullptr;    // per chunk: K of the adjoint's pair-mean part or S of the harmonic linear term

@@ -51,3 +51,23 @@ def test_pair_mean_table_leaves_the_kept_sums(prec, table, tmp_path):
     assert torch.equal(plan.cubic_retained(a, use_linear=True), ref)
     plan.sync()
     plan.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16x3"])
+@pytest.mark.parametrize("others", [1, NB, 7])
+def test_synthesis_of_other_maps_between(prec, others, tmp_path):
+    """modal_synthesize writes the caller's maps and leaves the kept ones, but goes through the Legendre sums."""
+    plan, files, sims, a, ref = _setup(prec, tmp_path)
+    plan.set_retain_maps(True)
+    b = torch.from_numpy(simgen.gaussian_alm(simgen.cl_model(L), others, seed=5).astype(np.complex64)).cuda()
+    plan.load_state(files["pixel"])
+    plan.cubic(a)
+    maps = plan.synthesize(b)
+    plan.cubic_retained(a, use_linear=True)                # per pixel: needs the maps alone
+    plan.set_linear_mode("ring")
+    plan.load_state(files["ring"])
+    for _ in range(2):
+        assert torch.equal(plan.cubic_retained(a, use_linear=True), ref)
+    assert torch.equal(plan.synthesize(b), maps)
+    plan.sync()
+    plan.close()
