@@ -1689,7 +1689,15 @@ modal_status modal_batch_cubic(modal_batch_h bh, const void* const* alm, const i
                           std::equal(bh->key_alm.begin(), bh->key_alm.end(), alm) &&
                           std::equal(bh->key_B.begin(), bh->key_B.end(), B) &&
                           std::equal(bh->key_beta.begin(), bh->key_beta.end(), beta);
-        if (!same) {
+        // the captured launches overwrite the members' map workspaces, whatever they kept before;
+        // what they keep is known once the graph has been launched
+        auto forget = [&] {
+            for (size_t i = 0; i < n; ++i)
+                if (B[i] > 0) bh->plans[i]->kept_alm = nullptr;
+        };
+        if (same) {
+            forget();
+        } else {
             batch_drop_graph(bh);
             std::vector<int> prof(n);
             for (size_t i = 0; i < n; ++i) {
@@ -1700,6 +1708,7 @@ modal_status modal_batch_cubic(modal_batch_h bh, const void* const* alm, const i
             const modal_status r = batch_run(bh, alm, B, use_linear, beta);
             cudaGraph_t g = nullptr;
             const cudaError_t ce = cudaStreamEndCapture(bh->main, &g);
+            forget();
             for (size_t i = 0; i < n; ++i) bh->plans[i]->prof = prof[i];
             if (r != MODAL_OK) {
                 if (g) cudaGraphDestroy(g);
@@ -1722,6 +1731,7 @@ modal_status modal_batch_cubic(modal_batch_h bh, const void* const* alm, const i
             bh->key_linear = use_linear ? 1 : 0;
         }
         CK(cudaGraphLaunch(bh->exec, bh->main), "graph launch");
+        for (size_t i = 0; i < n; ++i) keep_maps_if_whole(bh->plans[i], alm[i], B[i]);
     }
     CK(cudaEventRecord(bh->out, bh->main), "batch out");
     CK(cudaStreamWaitEvent(st, bh->out, 0), "batch out wait");

@@ -71,3 +71,30 @@ def test_synthesis_of_other_maps_between(prec, others, tmp_path):
     assert torch.equal(plan.synthesize(b), maps)
     plan.sync()
     plan.close()
+
+
+@pytest.mark.parametrize("schedule", ["streams", "shared_cubic"])
+def test_replayed_batch_replaces_the_kept_maps(schedule, tmp_path):
+    """A replay of a batch's graph writes its members' maps like the call that captured it: what another call kept before
+    is gone, what the batch synthesised is kept."""
+    plan, files, sims, a, ref = _setup("fp16x3", tmp_path)
+    import paper_1105_2791_gb300 as M
+    other = M.Plan(16, P, simgen.shifted_legendre_basis(16, P), simgen.cl_model(16), 17, NPHI)
+    c = torch.from_numpy(simgen.gaussian_alm(simgen.cl_model(16), 2, seed=6).astype(np.complex64)).cuda()
+    for p in (plan, other):
+        p.set_retain_maps(True)
+    batch = M.Batch([plan, other], schedule=schedule)
+    alms = [sims, c]
+    want = [b.clone() for b in batch.cubic(alms)]
+    assert torch.equal(plan.cubic_retained(sims), want[0])
+    plan.cubic(a)
+    for b, w in zip(batch.cubic(alms), want):              # the captured graph again
+        assert torch.equal(b, w)
+    with pytest.raises(M.ModalError) as e:
+        plan.cubic_retained(a)
+    assert e.value.status == M.MODAL_ESTATE
+    assert torch.equal(plan.cubic_retained(sims), want[0]) and torch.equal(other.cubic_retained(c), want[1])
+    plan.sync()
+    batch.close()
+    plan.close()
+    other.close()
