@@ -353,37 +353,52 @@ k_pair_ring_maps(int P, int nphi, int64_t npix, int nrings, int n_pair, const fl
 
 // h[b][(ab)][(cd)] = sum_j W_j <ab>_j rq[b][(cd)][j] (scale 1, rq of map b), and the two-pair sums
 // kmat[(ab)][(cd)] = sum_j nphi W_j <ab>_j <cd>_j (scale nphi, the means themselves as rq): FP64
-// products over the rings.  An FP64 instruction takes a warp 64 clocks whatever its lanes, so the
-// lanes hold rings (every one a useful product, contiguous reads), a warp eight (cd) of one (ab),
-// and the eight partial sums are added up across the warp in nine instructions instead of
-// forty.  With 8 rows per CTA and a thread per (cd), 8 maps at l_max = 300 with 10 modes took
-// 135 us (and the two-pair sums, a thread per pair, 102), now 35 (and 18).
-constexpr int QH_CD = 8;                                     // (cd) per warp
+// products over the rings.  An FP64 instruction takes a warp 64 clocks whatever its lanes, an SM's
+// warps together one per 19, so few sums are bound by the length of a warp's chain and many by the
+// number of instructions.  J lanes hold every J-th ring of one (ab) and eight (cd).  J = 32 (a warp
+// per (ab) and eight (cd)) has the shorter chain: 8 maps at l_max = 300 with 10 modes, 135 us with a
+// thread per (cd) and 8 rows per CTA, 35.  J = 8 (four neighbouring (ab) of the same (cd), whose
+// rows they read together) wastes fewer lanes on the last rings and on adding up, and takes its
+// weights W_j <ab>_j from a table instead of one more product per ring.  All per-ring terms of 500
+// maps, 61 rings, us with a thread per (cd) / J = 32 / J = 8: 16 modes 2585 / 3263 / 2414, 10 modes 1391 /
+// 676 / 594; 64 maps, 201 rings, 16 modes 1280 / 1313 / 1074; 64 maps, 21 rings 168 / 253 / 148.
+constexpr int QH_CD = 8;                                     // (cd) per lane
 constexpr int QH_WARPS = 4;
 
+__global__ void k_quartic_weights(int n, int nrings, int nphi, const double* __restrict__ mean, const float* __restrict__ W,
+                                  double* __restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = (double)W[(int64_t)(i % nrings) * nphi] * mean[i];
+}
+
+// mean: with J = 8 the table of the weights.
+template <int J>
 __global__ void __launch_bounds__(QH_WARPS * 32)
 k_quartic_hring(int n_pair, int nrings, int nphi, double scale, const double* __restrict__ rq, const double* __restrict__ mean,
                 const float* __restrict__ W, double* __restrict__ h) {
-    const int lane = threadIdx.x % 32, ab = blockIdx.x, b = blockIdx.z;
-    const int c0 = (blockIdx.y * QH_WARPS + threadIdx.x / 32) * QH_CD;
-    if (c0 >= n_pair) return;
+    const int lane = threadIdx.x % 32, jl = lane % J, b = blockIdx.y;
+    const int nchunk = (n_pair + QH_CD - 1) / QH_CD, ntask = n_pair * nchunk;
+    const int t0 = (blockIdx.x * QH_WARPS + threadIdx.x / 32) * (32 / J), t = t0 + lane / J;
+    if (t0 >= ntask) return;
+    const bool live = t < ntask;
+    const int ab = !live ? 0 : J == 32 ? t / nchunk : t % n_pair, c0 = !live ? 0 : (J == 32 ? t % nchunk : t / n_pair) * QH_CD;
     const double* m = mean + (int64_t)ab * nrings;
     const double* r = rq + ((int64_t)b * n_pair + c0) * nrings;
     double acc[QH_CD];
 #pragma unroll
     for (int i = 0; i < QH_CD; ++i) acc[i] = 0.0;
-    for (int j = lane; j < nrings; j += 32) {
+    for (int j = jl; j < nrings; j += J) {
         double v[QH_CD];
 #pragma unroll
         for (int i = 0; i < QH_CD; ++i) v[i] = c0 + i < n_pair ? r[(int64_t)i * nrings + j] : 0.0;
-        const double w = (double)W[(int64_t)j * nphi] * m[j];
+        const double w = J == 32 ? (double)W[(int64_t)j * nphi] * m[j] : m[j];
 #pragma unroll
         for (int i = 0; i < QH_CD; ++i) acc[i] = fma(w, v[i], acc[i]);
     }
-    // halves of the eight change places with the lane 16, 8 and 4 apart, then two plain steps:
-    // lane 4 i + k (any k) ends with the sum of (cd) c0 + index(i)
+    __syncwarp();
+    // halves of the eight change places with the lane J / 2, J / 4 and J / 8 apart, then plain steps
 #pragma unroll
-    for (int n = QH_CD / 2, o = 16; n >= 1; n /= 2, o /= 2) {
+    for (int n = QH_CD / 2, o = J / 2; n >= 1; n /= 2, o /= 2) {
         const bool up = lane & o;
 #pragma unroll
         for (int i = 0; i < n; ++i) {
@@ -391,17 +406,34 @@ k_quartic_hring(int n_pair, int nrings, int nphi, double scale, const double* __
             acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
-    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
-    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-    // bit 16 chose the upper four, bit 8 the upper two of these, bit 4 the upper one
-    const int cd = c0 + ((lane & 16) ? 4 : 0) + ((lane & 8) ? 2 : 0) + ((lane & 4) ? 1 : 0);
-    if (lane % 4 == 0 && cd < n_pair) h[((int64_t)b * n_pair + ab) * n_pair + cd] = scale * acc[0];
+#pragma unroll
+    for (int o = J / 16; o >= 1; o /= 2) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+    // bit J / 2 chose the upper four, bit J / 4 the upper two of these, bit J / 8 the upper one
+    const int cd = c0 + ((jl & (J / 2)) ? 4 : 0) + ((jl & (J / 4)) ? 2 : 0) + ((jl & (J / 8)) ? 1 : 0);
+    if (live && jl % (J / 8) == 0 && cd < n_pair) h[((int64_t)b * n_pair + ab) * n_pair + cd] = scale * acc[0];
 }
 
 static cudaError_t quartic_ring_products(Plan& pl, int B, double scale, const double* rq, double* out, cudaStream_t st) {
-    const int np = pl.n_pair, per = QH_CD * QH_WARPS;
-    k_quartic_hring<<<dim3(np, (np + per - 1) / per, B), QH_WARPS * 32, 0, st>>>(np, pl.nrings, pl.nphi, scale, rq, pl.ring_mean,
-                                                                               pl.W, out);
+    const int np = pl.n_pair, ntask = np * ((np + QH_CD - 1) / QH_CD);
+    // clocks of a warp's chain (64 per FP64 instruction and 600 for a step's reads) and of all the warps
+    // of an SM (19 per instruction): ten instructions per step and nine to add up with J = 32, eight and
+    // eight with J = 8, which needs the table first (a launch).  The estimates are good to a fifth: one
+    // map of 1000 rings, 16 modes, 173 us with J = 32 and 311 with 8; 8 maps 732 and 788; 64 maps 5299 and 4520.
+    auto clocks = [&](int64_t warps, int64_t steps, int64_t each, int64_t sum) {
+        return steps * (64 * each + 600) + 19 * ((warps + pl.nsm - 1) / pl.nsm) * (steps * each + sum);
+    };
+    const int64_t tasks = (int64_t)ntask * B;
+    const bool narrow = 5 * (clocks((tasks + 3) / 4, (pl.nrings + 7) / 8, 8, 8) + 4000) < 4 * clocks(tasks, (pl.nrings + 31) / 32, 10, 9);
+    if (narrow) {
+        const int n = np * pl.nrings;
+        k_quartic_weights<<<(n + 255) / 256, 256, 0, st>>>(n, pl.nrings, pl.nphi, pl.ring_mean, pl.W, pl.qt.wmean);
+        note_launch(pl);
+        k_quartic_hring<8><<<dim3((ntask + 4 * QH_WARPS - 1) / (4 * QH_WARPS), B), QH_WARPS * 32, 0, st>>>(
+            np, pl.nrings, pl.nphi, scale, rq, pl.qt.wmean, pl.W, out);
+    } else {
+        k_quartic_hring<32><<<dim3((ntask + QH_WARPS - 1) / QH_WARPS, B), QH_WARPS * 32, 0, st>>>(
+            np, pl.nrings, pl.nphi, scale, rq, pl.ring_mean, pl.W, out);
+    }
     note_launch(pl);
     return cudaGetLastError();
 }

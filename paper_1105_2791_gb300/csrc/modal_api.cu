@@ -270,7 +270,7 @@ static void destroy_plan(modal_plan* pl) {
     dfree(pl->ring_sum); dfree(pl->ring_mean);
     dfree(pl->solve_ws); dfree(pl->d_err); dfree(pl->adj_pm); dfree(pl->adj_pm_blk);
     dfree(pl->qt.tiles); dfree(pl->qt.idx); dfree(pl->qt.modes); dfree(pl->qt.pa); dfree(pl->qt.pb);
-    dfree(pl->qt.partial); dfree(pl->qt.rq); dfree(pl->qt.h); dfree(pl->qt.k3); dfree(pl->qt.kmat);
+    dfree(pl->qt.partial); dfree(pl->qt.rq); dfree(pl->qt.h); dfree(pl->qt.k3); dfree(pl->qt.kmat); dfree(pl->qt.wmean);
     free_tc_tables(*pl);
     free_tc_adj_tables(*pl);
     for (auto& pe : pl->prof_pending) { cudaEventDestroy(pe.second.first); cudaEventDestroy(pe.second.second); }
@@ -872,6 +872,7 @@ static modal_status ensure_quartic(modal_plan* h) {
     if (!h->qt.tiles) {
         CK(quartic_tables(*h), "quartic tables");
         CK(dalloc(h, &h->qt.k3, (size_t)h->qt.n_quad), "quartic two-pair term");
+        CK(dalloc(h, &h->qt.wmean, (size_t)h->n_pair * h->nrings), "quartic ring weights");
         CK(dalloc(h, &h->qt.kmat, (size_t)std::max(h->lin_ksplit, 1) * h->n_pair * h->n_pair), "quartic two-pair sums");
     }
     if (h->qt.chunk == h->chunk && h->qt.ctas == h->cubic_ctas) return MODAL_OK;

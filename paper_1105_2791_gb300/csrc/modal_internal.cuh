@@ -81,6 +81,7 @@ struct QuarticState {
     int* pb = nullptr;            // [n_pair] lexicographic pair -> b
     double* partial = nullptr;    // [chunk][cubic_ctas][n_quad]
     double* rq = nullptr;         // [chunk][n_pair][nrings] ring sums of pair products
+    double* wmean = nullptr;      // [n_pair][nrings] W_j <ab>_j (ring mode, many maps)
     double* h = nullptr;          // single-pair term: ring [chunk][n_pair][n_pair] or pixel [ksplit][n_pair][chunk n_pair]
     double* kmat = nullptr;       // two-pair sums [ksplit or 1][n_pair][n_pair]
     double* k3 = nullptr;         // [n_quad] two-pair term
