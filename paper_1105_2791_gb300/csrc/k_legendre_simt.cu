@@ -132,14 +132,25 @@ static void legendre_simt_launch(const Plan& pl, const float2* alm, int B, float
 
 template <int PM>
 static cudaError_t legendre_simt_pm(const Plan& pl, const float2* alm, int B, float2* delta, cudaStream_t st) {
-    // as many of the block's warps along the maps as there are maps for; two maps per thread where
-    // their sums leave room for three warps per sub-partition (16 modes, 16 maps, l_max = 500:
-    // 971 us with one, 1153 with two; 10 modes 861 and 734)
-    constexpr int MB = PM <= 12 ? 2 : 1;
-    if (B == 1) legendre_simt_launch<PM, 1, 1>(pl, alm, B, delta, st);
-    else if (B <= MB) legendre_simt_launch<PM, MB, 1>(pl, alm, B, delta, st);
-    else if (B <= 2 * MB) legendre_simt_launch<PM, MB, 2>(pl, alm, B, delta, st);
-    else legendre_simt_launch<PM, MB, 4>(pl, alm, B, delta, st);
+    if (B == 1) {
+        legendre_simt_launch<PM, 1, 1>(pl, alm, B, delta, st);
+    } else if constexpr (PM > 12) {
+        // the sums of two maps leave no room for three warps per sub-partition (16 modes, 16 maps,
+        // l_max = 500: 971 us with one per thread, 1153 with two; 10 modes 861 and 734)
+        if (B == 2) legendre_simt_launch<PM, 1, 2>(pl, alm, B, delta, st);
+        else legendre_simt_launch<PM, 1, 4>(pl, alm, B, delta, st);
+    } else {
+        // Two maps per thread from two warps per sub-partition on; below that the longer chain per
+        // order shows (10 modes, 8 maps, l_max = 32 9.7 us with two, 8.2 with one).  Four of a block's warps along the maps (eight maps, which read the table
+        // once), or two where that leaves an eighth fewer places empty: 9 maps of 10 modes, l_max =
+        // 250 104 and 95 us, l_max = 500 635 and 489 (12 maps 673 and 522); 16 maps, l_max = 250 126 and 134.
+        const int64_t warps = (int64_t)((pl.R_half + 31) / 32) * ((B + 1) / 2) * (pl.lmax + 1);
+        const int four = (B + 7) / 8 * 8, two = (B + 3) / 4 * 4;
+        if (warps < 8 * (int64_t)pl.nsm) legendre_simt_launch<PM, 1, 2>(pl, alm, B, delta, st);
+        else if (B == 2) legendre_simt_launch<PM, 2, 1>(pl, alm, B, delta, st);
+        else if (8 * two < 7 * four) legendre_simt_launch<PM, 2, 2>(pl, alm, B, delta, st);
+        else legendre_simt_launch<PM, 2, 4>(pl, alm, B, delta, st);
+    }
     return cudaGetLastError();
 }
 
