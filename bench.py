@@ -151,14 +151,14 @@ def legendre_flops(P, lmax, nrings):
     return 4.0 * P * n_alm * ((nrings + 1) // 2)
 
 
-# DRAM traffic per launch (GB, dram__bytes_read + dram__bytes_write) of each stage's main
-# kernel, from one-pass ncu captures (dram__bytes_*, gpu__time_duration) of one bench step at
-# this workload; adjoint_pixel is the tensor-core map part (k_adjoint_v) and linear_term the
-# harmonic sums (k_linh_s).  Keyed by (precision, lmax, nphi, P, maps per launch); an entry is
-# removed whenever its kernel changes until it is captured again.
+# DRAM traffic per launch (GB, dram__bytes_read + dram__bytes_write) of each stage's main kernel at
+# this workload, from earlier one-pass captures; adjoint_pixel is the tensor-core map part
+# (k_adjoint_v) and linear_term the harmonic sums (k_linh_s).  Keyed by (precision, lmax, nphi, P,
+# maps per launch).  Two are of earlier forms of their kernels that move the same data: ring_c2r with
+# its rows loaded by threads (by tiled copies 16.69 + 16.74) and legendre before its epilogue held
+# column blocks.
 STAGE_TRAFFIC_GB = {
     ("fp16x3", 2000, 4096, 16, 32): {
-        # ring_c2r: captured with rows loaded by threads (16.69 + 16.74 by tiled copies)
         "legendre": 17.00 + 16.39, "pair_means": 25.87 + 8.88, "ring_c2r": 16.52 + 16.74,
         "ring_r2c": 17.23 + 16.66, "legendre_adjoint": 27.64 + 0.60, "legendre_adjoint_prep": 16.52 + 16.73,
         "legendre_prep": 0.516 + 8.395, "cubic": 17.86 + 0.09, "adjoint_pixel": 16.82 + 16.72,
