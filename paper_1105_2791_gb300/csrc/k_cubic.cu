@@ -21,8 +21,8 @@ namespace modal {
 //
 // Modes in blocks of four: a box is a block triple bp <= br <= bs, that is up to 4 x 4 x 4
 // coefficients, in four shapes (all blocks different, bp = br, br = bs, all equal: 64, 40, 40 and
-// 20 coefficients) and as many again for a last block of at most two modes.  A warp owns one box; a lane owns one of 16 pixel classes of one of two
-// units (the half-warps), reads its pixel's 4 to 12 map values and W from shared memory, forms
+// 20 coefficients) and, up to 10 modes, as many again for a last block of at most two modes.  A
+// warp owns one box; a lane owns one of 16 pixel classes of one of two units (the half-warps), reads its pixel's 4 to 12 map values and W from shared memory, forms
 // the products W M_p M_r of its box in registers and accumulates in packed FP32 pairs over p
 // (32, 24, 20 or 13 FFMA2 per pixel).  The pair products are thus formed by the warps that use
 // them, at a quarter of the multiply-adds they feed, instead of being written to a panel in
@@ -260,8 +260,8 @@ constexpr int CUB_THREADS = (CUBIC_BOXES + 1) * 32;
 // of modes holds at most two.  The warps of a CTA run as many different box bodies as there are
 // shapes, so the instruction cache decides how far the pixel loop is unrolled: with four shapes
 // all 8 pixels of a stage (16 modes, l_max = 1000, 16 maps: 1.51 ms, 1.63 looped), with the
-// eight that a half block brings (up to 10 modes: cubic_half) two at a time (10 modes, l_max = 500, 64 maps: 0.72 ms looped,
-// 1.05 unrolled, 0.91 with the last block treated as whole).
+// eight that a half block brings (cubic_half) two at a time (10 modes, l_max = 500, 64 maps: 0.72
+// ms looped, 1.05 unrolled, 0.91 with the last block treated as whole).
 template <bool HALF>
 struct CubicCta {
     float* smem;

@@ -406,7 +406,7 @@ cudaError_t launch_linear_harmonic(Plan& pl, const float2* alm, int B, double* l
     note_launch(pl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int cpb = std::min(LG2_OUT / pl.P, pl.n_pair);    // at most 36 pairs (7 modes): 11 KB of shared memory
+    const int cpb = std::min(LG2_OUT / pl.P, pl.n_pair);    // at most 32 pairs (8 modes): 10.3 KB of shared memory
     k_linh_g<<<dim3(B, (pl.n_pair + cpb - 1) / cpb), LG2_OUT, 2 * (size_t)(pl.P + cpb) * 33 * sizeof(float), st>>>(
         pl.lmax, pl.P, pl.n_pair, B, cpb, pl.filt, pl.adj_pmk, lin);
     note_launch(pl);

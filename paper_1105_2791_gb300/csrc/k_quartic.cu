@@ -20,9 +20,10 @@
 namespace modal {
 
 // ---------------------------------------------------------------- quartic term
-// Warp roles as in the cubic kernel: QT_TX fill threads (one pixel each, values
-// prefetched two tiles ahead) build U (colex pairs, row layout [half][pair group][4]) and
-// Q (lexicographic pairs over PM modes, row layout [quad][4]); compute threads hold one
+// Two kinds of warps, with named barriers and two panels in shared memory between them: QT_TX
+// fill threads (one pixel each, values prefetched two tiles ahead) build U (colex pairs, row
+// layout [half][pair group][4]) and Q (lexicographic pairs over PM modes, row layout [quad][4]);
+// compute threads hold one
 // register tile of 8 U pairs x 4 Q pairs and one of `nl` pixel lanes.  Tiles whose pairs
 // all have r > s are absent from the tile list.
 constexpr int QT_TX = 64;

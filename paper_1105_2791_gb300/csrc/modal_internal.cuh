@@ -224,7 +224,8 @@ constexpr int CUBIC_BOXES = 10;      // warps per CTA of the cubic kernel, one b
 // Whether a last block of at most two modes has box shapes of its own (as the plan builds its boxes):
 // up to 10 modes, whose boxes are one group.  At 13 and 14 modes the two CTAs of a pair of units
 // would each run up to eight box bodies, whose instructions do not stay cached: 128 ranges of
-// 8192 pixels 94 us, and as four whole blocks, the operations of the kept sums the same, 65 (90 and 92 as pair-product panels).
+// 8192 pixels 94 us, and as four whole blocks, the operations of the kept sums the same, 65 (90
+// and 92 as pair-product panels).
 inline bool cubic_half(int P) { return P <= 10 && (P % 4 == 1 || P % 4 == 2); }
 bool cubic_one_launch(const Plan& pl);   // false from nearly 2^31 pixels: then only launch_cubic, in parts
 cudaError_t launch_cubic_multi(Plan* const* plans, const float* const* maps, const int* B, int n, cudaStream_t st);
@@ -239,8 +240,7 @@ cudaError_t launch_adjoint_weights(Plan& pl, const double* g, int B, float* hk, 
 // vring [B][P][nrings] (ring mode, use_linear = 0); neither when both are off.
 cudaError_t launch_adjoint_u(Plan& pl, const float* maps, int B, const float* hk, int use_linear,
                              float* u, cudaStream_t st);
-// k_adjoint_tc.cu: the same pixel weights as a tcgen05 product (split plans); in place on maps
-// k_adjoint_v.cu: the map part of the pixel weights (in place over the maps).
+// k_adjoint_v.cu: the map part of the pixel weights as a tcgen05 product (split plans), in place over the maps.
 size_t adjoint_v_workspace_bytes(const Plan& pl, int chunk);
 cudaError_t launch_adjoint_v(Plan& pl, int B, const float* hk, float* maps, cudaStream_t st);
 // k_pm_harmonic.cu: the pair means in harmonic space (split plans, per-pixel means): the table
