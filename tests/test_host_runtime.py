@@ -19,7 +19,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 def host_library(tmp_path_factory):
     build.build()
     out = str(tmp_path_factory.mktemp("host") / "libmodal_host.so")
-    cuda = os.path.dirname(os.path.dirname(build.nvcc()))
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc())))
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I" + os.path.join(cuda, "include"),
                     "-I" + build.CSRC, os.path.join(HERE, "host_runtime", "fake_runtime.cpp")] +
                    sorted(glob.glob(os.path.join(build.BUILD, "*.o"))) + ["-o", out], check=True)
